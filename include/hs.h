@@ -69,8 +69,10 @@ typedef struct {
   int pad;
 } hs_minres_info;
 
-/* Solver forms (all run the recurrence of Algorithm 2): vectors resident in
- * shared memory (chains up to L = 20 in FP64, 22 in FP32); superblock passes
+/* Solver forms (all run the recurrence of Algorithm 2): vectors resident on
+ * chip (HS_FORM_SMEM: one thread-block cluster for chains of up to 16384 rows,
+ * in FP64 up to 4096, else shared memory of the whole grid, chains up to
+ * L = 20 in FP64, 22 in FP32); superblock passes
  * (from L = 24 on); one persistent cooperative kernel with vectors in global
  * memory; per-pass kernels replayed from a CUDA graph; and the shared-memory
  * form with one global reduction per iteration (the product taken of

@@ -710,6 +710,17 @@ static bool pipe_choice(const hs_handle* hd, bool f64, int pc) {
   return hd->n <= 1024LL * G;
 }
 
+// The cluster form (minres_clu.cu) takes the small solves. Not where another
+// form is asked for (HS_MINRES_PIPE), nor under HS_BARRIER_LIMIT, which limits
+// the waits of the grid forms. HS_MINRES_CLUSTER=0 turns it off.
+static int cluster_choice(const hs_handle* hd, bool f64, int pc) {
+  if (getenv("HS_MINRES_PIPE") || getenv("HS_BARRIER_LIMIT")) return 0;
+  // FP64 above 4096 rows: 16 SMs' FP64 pipes would bound it
+  if (f64 && hd->n > 4096 && pipe_choice(hd, f64, pc)) return 0;
+  const int bud = hd->sm_budget.load(std::memory_order_relaxed);
+  return clu_choice(hd->n, std::max(1, std::min(hd->num_sms, bud > 0 ? bud : hd->num_sms)));
+}
+
 template <typename T, int PC>
 static hs_status try_sb(hs_handle* hd, const T* b, const MinresVecs& v, double tol,
                         long long kmax) {
@@ -729,6 +740,11 @@ static hs_status solve_pc(hs_handle* hd, const T* b, T* x, double tol, long long
   int form = 0;
   const int sbc = sb_choice(hd);
   if (sbc == 2 && (st = try_sb<T, PC>(hd, b, v, tol, kmax)) != HS_CUDA) form = HS_FORM_SUPERBLOCK;
+  const int cs = st == HS_CUDA && !force_graph() && !force_global()
+                     ? cluster_choice(hd, sizeof(T) == 8, PC) : 0;
+  if (cs > 0 && (st = solve_clu(hd, b, v.x, sizeof(T) == 8 ? HS_F64 : HS_F32, PC, tol, kmax,
+                                cs)) != HS_CUDA)
+    form = HS_FORM_SMEM;
   if (st == HS_CUDA && !force_graph() && !force_global() && pipe_choice(hd, sizeof(T) == 8, PC) &&
       (st = solve_smem_job(hd, b, v, sizeof(T) == 8 ? HS_F64 : HS_F32, PC, tol, kmax, true)) !=
           HS_CUDA)

@@ -1,0 +1,99 @@
+// Preconditioned MINRES of Algorithm 2 (Appendix A) in one thread-block
+// cluster, for chains of up to 16384 rows (minres_clu.cuh): the kernel of a
+// single solve and the choice of the cluster size.
+#include <algorithm>
+#include <cstdlib>
+
+#include "minres_clu.cuh"
+
+namespace hs {
+
+namespace {
+
+template <typename T, int RPT>
+__global__ void __launch_bounds__(CLU_NT, 1) k_minres_clu(SmemJob job, int pc) {
+  extern __shared__ __align__(16) char dyn[];
+  __shared__ CluShared sh;
+  clu_setup(sh);
+  CluPhase ph;
+  clu_solve<T, RPT>(job, pc, sh, dyn, ph);
+  clu_sync();   // no CTA leaves while another may still write to it
+}
+
+template <typename T, int RPT>
+hs_status launch_t(hs_handle* hd, const SmemJob& job, int pc, int cs) {
+  const size_t sm = clu_bytes<T>((int)hd->n, hd->L, cs, RPT);
+  auto kern = k_minres_clu<T, RPT>;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(cs);
+  cfg.blockDim = dim3(CLU_NT);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = hd->stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cs;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) !=
+          cudaSuccess ||
+      (cs > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+                     cudaSuccess) ||
+      cudaLaunchKernelEx(&cfg, kern, job, pc) != cudaSuccess) {
+    cudaGetLastError();
+    return HS_CUDA;
+  }
+  count_launches(1);
+  return HS_OK;
+}
+
+template <typename T>
+hs_status launch_rpt(hs_handle* hd, const SmemJob& job, int pc, int cs) {
+  const int rpc = ((int)hd->n + cs - 1) / cs;
+  const int rpt = (rpc + 32 * CLU_NW - 1) / (32 * CLU_NW);
+  // rows per thread: as few as hold the rows in FP64 (each row is FP64 work on
+  // the critical path); two at least in FP32, where half the warps make half
+  // the partials and messages (n = 924, 8 CTAs: 1.72 -> 1.59 us per iteration;
+  // FP64 there 2.38 -> 3.00)
+  if constexpr (sizeof(T) == 8)
+    if (rpt <= 1) return launch_t<T, 1>(hd, job, pc, cs);
+  if (rpt <= 2) return launch_t<T, 2>(hd, job, pc, cs);
+  if (rpt <= 4) return launch_t<T, 4>(hd, job, pc, cs);
+  if (rpt <= CLU_RPT_MAX) return launch_t<T, CLU_RPT_MAX>(hd, job, pc, cs);
+  return HS_CUDA;
+}
+
+}  // namespace
+
+// CTAs per cluster. More CTAs share the FP64 work but make every exchange
+// longer. Measured per iteration (us, row norm, FP64 / FP32; the grid forms
+// that took these solves before in brackets):
+//   n = 70     1 CTA 1.83 / 1.05, 8 CTAs 1.82 / 1.4                     (12.2 / 15.2)
+//   n = 252    1 CTA 2.73 / 1.38, 2 CTAs 2.10 / 1.35, 8 CTAs 2.02 / 1.48  (11.4 / 15.6)
+//   n = 924    4 CTAs 3.13 / 1.60, 8 CTAs 2.38 / 1.59, 16 CTAs 2.34 / 1.65 (11.7 / 15.6)
+//   n = 3432   8 CTAs 5.4 / 2.4, 16 CTAs 4.12 / 2.16                       (12.2 / 17.1)
+//   n = 12870  16 CTAs FP32 4.98                                            (17.8)
+// FP64 at n = 12870 stays with the grid forms (pipe_choice). HS_MINRES_CLUSTER
+// sets the number of CTAs (a power of two, at most 16; 0: off).
+int clu_choice(long long n, int sms) {
+  if (n > CLU_ROWS_MAX) return 0;
+  int cs = n <= 128 ? 1 : n <= 512 ? 2 : n <= 1024 ? 8 : 16;
+  if (const char* e = getenv("HS_MINRES_CLUSTER")) cs = atoi(e);
+  while (cs > sms) cs >>= 1;
+  return cs;
+}
+
+hs_status solve_clu(hs_handle* hd, const void* b, void* x, hs_dtype dt, int pc, double tol,
+                    long long kmax, int cs) {
+  const SmemJob job{hd->geo(), b, x, hd->d_state, hd->sigma, tol, kmax};
+  const hs_status st = dt == HS_F64 ? launch_rpt<double>(hd, job, pc, cs)
+                                    : launch_rpt<float>(hd, job, pc, cs);
+  if (st != HS_OK) return st;
+  HS_CUDA_TRY(hd, cudaMemcpyAsync(hd->h_state, hd->d_state, sizeof(MinresState),
+                                  cudaMemcpyDeviceToHost, hd->stream));
+  HS_CUDA_TRY(hd, cudaStreamSynchronize(hd->stream));
+  return HS_OK;
+}
+
+}  // namespace hs

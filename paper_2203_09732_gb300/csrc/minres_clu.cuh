@@ -1,0 +1,538 @@
+// Preconditioned MINRES of Algorithm 2 (Appendix A) inside one thread-block
+// cluster, for chains of up to 16384 rows: the device side, shared by the
+// single solve (minres_clu.cu) and the batched sweep (sweep.cu).
+//
+// What bounds a small solve is latency: two reductions per iteration over all
+// rows, and the FP64 pipe, which takes 64 cycles per warp instruction and SM
+// quarter whatever the number of active lanes (measured: dependent or not, 1
+// lane or 32). So:
+//   * the CTAs of a cluster exchange through distributed shared memory: every
+//     warp sends its partial sum to every CTA (st.async, counted by an mbarrier
+//     in the receiving CTA, about 450 cycles), no grid barrier and no trip
+//     through L2 (about 2500 cycles a reduction in the grid forms);
+//   * every CTA holds a full copy of q; the owner of a row sends the new entry
+//     to all copies the same way, so the product's gathers are shared-memory
+//     loads from per-row neighbour lists;
+//   * a thread owns RPT rows for the whole solve and keeps their vectors in
+//     registers: CLU_NW compute warps, one per SM quarter, saturate the FP64 pipe;
+//   * three control warps per CTA take the scalars off the compute warps' path:
+//     one adds the partials of alpha_k and forms the coefficient that needs it,
+//     one adds those of beta_k^2 and has 1 / beta_k and its powers ready by then,
+//     one runs the Givens rotation of Algorithm 2 an iteration behind; the compute
+//     warps apply its d/x update two iterations behind, while they wait for
+//     alpha. Where several scalars need the same operation, each takes a lane.
+// All CTAs sum the same numbers in the same order, so they hold identical
+// scalars and take the same branches.
+#pragma once
+#include "minres_smem.cuh"
+
+namespace hs {
+
+constexpr int CLU_NW = 4;                       // compute warps per CTA
+constexpr int CLU_CW = 3;                       // control warps (warps 0, 1 and 2)
+constexpr int CLU_NT = 32 * (CLU_NW + CLU_CW);
+constexpr int CLU_SIZE_MAX = 16;                // CTAs per cluster
+constexpr int CLU_RPT_MAX = 8;                  // rows per thread
+constexpr int CLU_ROWS_MAX = CLU_SIZE_MAX * 32 * CLU_NW * CLU_RPT_MAX;
+// polls of an mbarrier before a wait gives up with HS_TIMEOUT
+constexpr unsigned CLU_WAIT_LIMIT = 1u << 22;
+
+// Exchange words of one CTA (shared memory). What one warp hands to a later
+// iteration of another has two places, used in turn.
+struct CluShared {
+  double slotA[CLU_SIZE_MAX * CLU_NW];          // partials of alpha_k
+  double slotB[CLU_SIZE_MAX * CLU_NW];          // partials of beta_{k+1}^2
+  unsigned long long barA, barB;                // remote data of the two phases
+  unsigned long long barC;                      // alpha warp -> compute warps
+  unsigned long long barF[2];                   // beta warp -> alpha warp
+  unsigned long long barE[2];                   // alpha warp -> rotation warp
+  unsigned long long barD[2];                   // rotation warp -> the others
+  double c[3];                                  // coefficients of q_{k+1}, of type T
+  double f[2][8];                               // F: sum = beta_k^2, beta_k, 1/beta_{k-1}, 1/beta_k,
+                                                //    1/(2 beta_k^2), 1/(2 beta_k^3), beta_k/beta_{k-1}
+  double alpha[2];                              // E: alpha_k
+  struct { double co[4]; int apply, stop; } d[2];   // D: cq, cd1, cd2, tau (of type T)
+  int fail;
+  MinresState S;                                // the solve's state (rotation warp)
+};
+
+__device__ __forceinline__ uint32_t smem_u32(const void* p) {
+  return (uint32_t)__cvta_generic_to_shared(p);
+}
+__device__ __forceinline__ uint32_t clu_map(uint32_t addr, uint32_t cta) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(cta));
+  return r;
+}
+__device__ __forceinline__ void clu_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n"
+               "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t clu_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t clu_size() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void bar_init(unsigned long long* b, unsigned count) {
+  asm volatile("mbarrier.init.shared.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void bar_arm(unsigned long long* b, unsigned bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void bar_arrive(unsigned long long* b) {
+  asm volatile("mbarrier.arrive.shared.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
+}
+// Waits for the phase of the given parity; false after CLU_WAIT_LIMIT polls.
+__device__ __forceinline__ bool bar_wait(unsigned long long* b, unsigned parity) {
+  const uint32_t a = smem_u32(b);
+  for (unsigned it = 0; it < CLU_WAIT_LIMIT; ++it) {
+    uint32_t done;
+    asm volatile("{\n.reg .pred p;\n"
+                 "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+                 "selp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(done) : "r"(a), "r"(parity) : "memory");
+    if (done) return true;
+  }
+  return false;
+}
+// One or two values into another CTA's shared memory, counted by its mbarrier.
+__device__ __forceinline__ void clu_send(uint32_t dst, double v, uint32_t bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(dst),
+               "l"(__double_as_longlong(v)), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void clu_send(uint32_t dst, float v, uint32_t bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(dst),
+               "r"(__float_as_uint(v)), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void clu_send2(uint32_t dst, double v, double w, uint32_t bar) {
+  asm volatile(
+      "st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(dst),
+      "l"(__double_as_longlong(v)), "l"(__double_as_longlong(w)), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void clu_send2(uint32_t dst, float v, float w, uint32_t bar) {
+  asm volatile(
+      "st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(dst),
+      "r"(__float_as_uint(v)), "r"(__float_as_uint(w)), "r"(bar) : "memory");
+}
+template <typename T>
+__device__ __forceinline__ T warp_sum_all(T v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Rows per CTA. With two or more rows a thread holds pairs of consecutive rows
+// (one message per pair and copy: sending costs by the message), pair i of
+// thread t at 2 (128 i + t): wider runs per thread would put the lanes of a
+// gather on the same banks. Rows past n (in the last CTAs) are sent as zeros.
+__host__ __device__ inline int clu_rows(int n, int cs, int rpt) {
+  const int r = (n + cs - 1) / cs;
+  return rpt == 1 ? r : (r + 1) & ~1;
+}
+// Dynamic shared memory of a CTA: the copy of q with one zero element behind
+// it, then the neighbour lists (pairs of 16-bit row numbers, [pair][j][thread]).
+template <typename T>
+__host__ __device__ inline size_t clu_q_bytes(int n, int cs, int rpt) {
+  return (((size_t)cs * clu_rows(n, cs, rpt) + 1) * sizeof(T) + 15) & ~size_t(15);
+}
+template <typename T>
+__host__ __device__ inline size_t clu_bytes(int n, int L, int cs, int rpt) {
+  return clu_q_bytes<T>(n, cs, rpt) + sizeof(uint32_t) * (size_t)(L / 2) * 32 * CLU_NW * rpt;
+}
+
+// Phase parities of a cluster's barriers, carried from solve to solve.
+struct CluPhase {
+  unsigned a = 0, b = 0, c = 0, d[2] = {0, 0}, e[2] = {0, 0}, f[2] = {0, 0};
+};
+
+// Barriers of a CTA, once per kernel, before the first solve (all threads).
+__device__ __forceinline__ void clu_setup(CluShared& sh) {
+  if (threadIdx.x == 0) {
+    bar_init(&sh.barA, 1);
+    bar_init(&sh.barB, 1);
+    bar_init(&sh.barC, 1);
+    for (int i = 0; i < 2; ++i) {
+      bar_init(&sh.barF[i], 1);
+      bar_init(&sh.barE[i], 1);
+      bar_init(&sh.barD[i], 1);
+    }
+    sh.fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  clu_sync();
+}
+
+// Sum of the np partials of all warps of the cluster, in every lane.
+__device__ __forceinline__ double clu_total(const double* slot, int np) {
+  const int lane = threadIdx.x & 31;
+  double v = lane < np ? slot[lane] : 0.0;
+  if (np > 32) v += lane + 32 < np ? slot[lane + 32] : 0.0;
+  // a tree over the lanes that hold partials only: each level costs an FP64 add
+  for (int o = np > 16 ? 16 : np > 8 ? 8 : np > 4 ? 4 : np > 2 ? 2 : np > 1 ? 1 : 0; o > 0; o >>= 1)
+    v += __shfl_xor_sync(0xffffffffu, v, o);
+  return __shfl_sync(0xffffffffu, v, 0);
+}
+static_assert(CLU_SIZE_MAX * CLU_NW <= 64, "clu_total adds two partials per lane");
+
+// The Givens rotation of step k (Algorithm 2) and its d/x coefficients: the
+// quantities of givens_fast, with a reciprocal square root instead of a root
+// and divisions, and one lane per scalar where the operation is the same
+// (every lane computes; lanes past the first few repeat them). sumsq =
+// beta_{k+1}^2, bn = beta_{k+1}, ib = 1 / beta_k.
+__device__ __forceinline__ void clu_givens(MinresState& S, double sumsq, double bn, double ib) {
+  constexpr unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 7;
+  const double cp = S.c_prev, sp = S.s_prev;
+  // lane 0: delta_k = c dh + s alpha; lane 1: hat gamma_k = c alpha - s dh
+  const double u = lane & 1 ? S.alpha : S.delta_hat, w = lane & 1 ? -S.delta_hat : S.alpha;
+  const double r = cp * u + sp * w;
+  const double delta = __shfl_sync(full, r, 0), gh = __shfl_sync(full, r, 1);
+  const double g2 = gh * gh + sumsq;                         // gamma_k^2
+  if (!isfinite(bn) || !isfinite(g2)) {
+    S.status = HS_NONFINITE; S.done = 2; S.pending = 0;
+    return;
+  }
+  if (g2 == 0.0) {
+    S.status = HS_BREAKDOWN; S.done = 2; S.pending = 0;
+    return;
+  }
+  const double rg = rsqrt(g2);
+  // times 1 / gamma_k: c_k, s_k, the three coefficients of d_k
+  const double v = lane == 0 ? gh : lane == 1 ? bn : lane == 2 ? ib : lane == 3 ? -delta : -S.eps;
+  const double t = v * rg;
+  const double c = __shfl_sync(full, t, 0), sn = __shfl_sync(full, t, 1);
+  S.cq = __shfl_sync(full, t, 2);
+  S.cd1 = __shfl_sync(full, t, 3);
+  S.cd2 = __shfl_sync(full, t, 4);
+  // tau_k = c phi, phi_k = -s phi, epsilon_{k+1} = s_{k-1} beta, hat delta_{k+1} = c_{k-1} beta
+  const double x = lane == 0 ? c : lane == 1 ? -sn : lane == 2 ? sp : cp;
+  const double y = x * (lane < 2 ? S.phi : bn);
+  S.tau = __shfl_sync(full, y, 0);
+  S.phi = __shfl_sync(full, y, 1);
+  S.eps = __shfl_sync(full, y, 2);
+  S.delta_hat = __shfl_sync(full, y, 3);
+  S.pending = 1;
+  S.beta_prev = S.beta; S.beta = bn;
+  S.c_prev = c; S.s_prev = sn;
+  S.k = S.k + 1;
+  if (fabs(S.phi) < S.tol_abs || bn == 0.0 || S.k > S.kmax) S.done = 1;
+}
+
+// One solve by one cluster; every thread of every CTA calls it with the same
+// job. Rows are dealt to the CTAs in contiguous runs of rank order. Returns
+// false when a wait gave up (status HS_TIMEOUT). The final state is in sh.S of
+// every CTA and, if job.st is set, in *job.st.
+//
+// Order of events (k = 1, 2, ...; the phases of a barrier follow each other
+// because each is complete only when every warp of the cluster has sent, and a
+// warp sends only after it has read what the phase before brought):
+//   compute   wait B (q_k); p_k = (H - sigma) q_k; send alpha partials (A);
+//             wait D (step k - 2): apply its d/x update, leave if it was the last;
+//             wait C: q_{k+1}; send it and its norm's partials (B)
+//   beta      wait B: beta_k and its reciprocal powers (F)
+//   alpha     wait A, F, D (step k - 2): leave if it was the last; C: the
+//             coefficients of q_{k+1}; E: alpha_k
+//   rotation  wait F (beta_k) and E (alpha_{k-1}): the rotation of step k - 1; D: its
+//             coefficients
+template <typename T, int RPT>
+__device__ bool clu_solve(const SmemJob& job, int pc, CluShared& sh, char* dyn, CluPhase& ph) {
+  const Geo& g = job.g;
+  const int n = (int)g.n;
+  const int cs = (int)clu_size(), me = (int)clu_rank();
+  const int lane = threadIdx.x & 31;
+  const int wid = (int)(threadIdx.x >> 5) - CLU_CW;   // compute warp, negative: control
+  constexpr int SLOTS = 32 * CLU_NW * RPT;
+  T* Q = reinterpret_cast<T*>(dyn);
+  uint32_t* nbr = reinterpret_cast<uint32_t*>(dyn + clu_q_bytes<T>(n, cs, RPT));
+  const int rpc = clu_rows(n, cs, RPT);
+  const int r0 = me * rpc, zero = cs * rpc;           // first row, the zero element
+  constexpr int V = RPT == 1 ? 1 : 2;                 // consecutive rows of a thread
+  const int nwa = min(CLU_NW, (rpc / V + 31) / 32);   // compute warps with rows
+  const int np = cs * nwa;
+  const unsigned bytesA = 8u * np, bytesB = 8u * np + (unsigned)sizeof(T) * zero;
+  const double sigma = job.sigma;
+  if (threadIdx.x == 0) Q[zero] = T(0);
+  clu_sync();                                    // every CTA has left the previous solve
+  // A barrier's bytes are announced just before the wait of the warp that owns
+  // it: data that came earlier has been counted (the count may be negative
+  // meanwhile), and the phase cannot complete without this arrival.
+  auto take = [&](unsigned long long* bar, unsigned bytes, unsigned& parity) {
+    if (lane == 0) bar_arm(bar, bytes);
+    __syncwarp();
+    const bool got = bar_wait(bar, parity);
+    parity ^= 1u;
+    return got;
+  };
+  if (wid >= 0 && wid < nwa) {
+    // ---- compute warps
+    T q[RPT], qm[RPT], ql[RPT];                  // q_k, q_{k-1}, q_{k-2}
+    T d1[RPT], d2[RPT], x[RPT], m[RPT], mi[RPT], dg[RPT];
+    int np2[RPT];                                // neighbour pairs of the warp's longest row
+    const int t0 = wid * 32 + lane;
+    auto lrow = [&](int j) { return ((j / V) * 32 * CLU_NW + t0) * V + j % V; };   // in the CTA
+    const uint32_t aBarA = smem_u32(&sh.barA), aBarB = smem_u32(&sh.barB);
+    const uint32_t aSA = smem_u32(&sh.slotA[me * nwa + wid]);
+    const uint32_t aSB = smem_u32(&sh.slotB[me * nwa + wid]);
+    const uint32_t aQ = smem_u32(Q + r0 + t0 * V);
+    auto slot_of = [&](int j) { return j * 32 * CLU_NW + t0; };
+    auto owned = [&](int j) { return lrow(j) < rpc && r0 + lrow(j) < n; };
+    T acc = T(0);
+    double zm = 0.0;
+#pragma unroll
+    for (int j = 0; j < RPT; ++j) {
+      const int slot = slot_of(j);
+      q[j] = qm[j] = ql[j] = d1[j] = d2[j] = x[j] = m[j] = mi[j] = dg[j] = T(0);
+      int cnt = 0;
+      if (owned(j)) {
+        const uint32_t i = (uint32_t)(r0 + lrow(j));
+        // the row's block: the last one that starts at or before it
+        int lo = 0, hi = g.nblocks - 1;
+        while (lo < hi) {
+          const int mid = (lo + hi + 1) >> 1;
+          if (__ldg(&g.blocks[mid].R) <= i) lo = mid;
+          else hi = mid - 1;
+        }
+        const uint32_t* bw = reinterpret_cast<const uint32_t*>(g.blocks + lo);
+        Hdr h;
+        h.R = __ldg(bw);
+        h.Rwrap = __ldg(bw + 1);
+        h.bdelta = (int32_t)__ldg(bw + 2);
+        const uint32_t meta = __ldg(bw + 3);
+        h.w = meta & 0xFF;
+        h.nh = (meta >> 8) & 0xFF;
+        h.code = (meta >> 16) & 0xFF;
+        h.off = g.cls_off[h.w];
+        h.dhs = __hiloint2double((int)__ldg(bw + 5), (int)__ldg(bw + 4)) - sigma;
+        h.dhs_f = (float)h.dhs;
+        const LowEntry e = g.low[h.off + (int)(i - h.R)];
+        const uint32_t xc = cut_mask(e.packed, h);
+        uint16_t* out = reinterpret_cast<uint16_t*>(nbr);
+        auto put = [&](uint32_t r) {
+          out[((cnt >> 1) * SLOTS + slot) * 2 + (cnt & 1)] = (uint16_t)r;
+          ++cnt;
+        };
+        for (int b = 0; b < le_cnt(e.packed); ++b)
+          put(h.R + ((e.nbw[b >> 2] >> (8 * (b & 3))) & 0xFFu));
+        for (int b = 0; b < h.nh; ++b) put((uint32_t)((int)i + (int)__ldg(bw + 6 + b)));
+        if (xc & 1u) put((uint32_t)((int)i + h.bdelta));
+        if (xc & 2u) put(h.Rwrap + e.wrap_r);
+        const T am = diag_t<T>(e, h, xc);
+        const int naf = naf_row(e.packed, h, xc);
+        const T mm = pc == 0 ? precond_t<0, T>(am, naf)
+                   : pc == 1 ? precond_t<1, T>(am, naf) : precond_t<2, T>(am, naf);
+        const T b = reinterpret_cast<const T*>(job.b)[i];
+        zm += mm == T(0) ? 1.0 : 0.0;
+        const T im = mm == T(0) ? T(0) : T(1) / mm;
+        q[j] = b * im;
+        m[j] = mm;
+        mi[j] = T(0.5) * im;                     // p is kept doubled, see below
+        dg[j] = T(2) * am;
+        acc += q[j] * b;
+      }
+      // a walk round the ring crosses an even number of antiparallel bonds
+      np2[j] = __reduce_max_sync(0xffffffffu, cnt >> 1);
+      for (int c = cnt >> 1; c < np2[j]; ++c)
+        nbr[c * SLOTS + slot] = (uint32_t)zero | (uint32_t)zero << 16;
+    }
+    // q_{k+1} to every copy and the partial of its norm
+    auto publish = [&](T part) {
+      if (lrow(0) < rpc) {
+#pragma unroll 4
+        for (int c = 0; c < cs; ++c) {
+          const int to = me + c < cs ? me + c : me + c - cs;
+          const uint32_t rq = clu_map(aQ, to), rb = clu_map(aBarB, to);
+#pragma unroll
+          for (int j = 0; j < RPT; j += V)
+            if (j == 0 || lrow(j) < rpc) {
+              const uint32_t d = rq + (uint32_t)(j * 32 * CLU_NW * sizeof(T));
+              if constexpr (V == 1) clu_send(d, q[j], rb);
+              else clu_send2(d, q[j], q[j + 1], rb);
+            }
+        }
+      }
+      const double s = (double)warp_sum_all(part);
+      if (lane < cs) clu_send(clu_map(aSB, lane), s, clu_map(aBarB, lane));
+    };
+    publish(acc);
+    zm = warp_sum_all(zm);
+    if (lane < cs) clu_send(clu_map(aSA, lane), zm, clu_map(aBarA, lane));
+    // step 0 of D: the initial state
+    bool ok = bar_wait(&sh.barD[0], ph.d[0]);
+    ph.d[0] ^= 1u;
+    bool run = ok && sh.d[0].stop == 0;
+    unsigned pb = ph.b;
+    for (int k = 1; run; ++k) {
+      if (!(ok = bar_wait(&sh.barB, pb))) break;   // q_k has arrived
+      pb ^= 1u;
+      // p_k, doubled: 2 (H - sigma) q = (2 a_ii - 2 sigma) q_i + sum over neighbours
+      T p[RPT];
+      acc = T(0);
+#pragma unroll
+      for (int j = 0; j < RPT; ++j) {
+        const uint32_t* nl = nbr + slot_of(j);
+        T s = T(0);
+#pragma unroll 4
+        for (int c = 0; c < np2[j]; ++c) {
+          const uint32_t w = nl[c * SLOTS];
+          s += Q[w & 0xFFFFu];
+          s += Q[w >> 16];
+        }
+        p[j] = dg[j] * q[j] + s;
+        acc += q[j] * p[j];
+      }
+      const double pa = (double)warp_sum_all(acc);
+      if (lane < cs) clu_send(clu_map(aSA, lane), pa, clu_map(aBarA, lane));
+      // d_{k-2} and x_{k-2} while alpha_k travels
+      if (k > 2) {
+        const int t = k & 1;
+        if (!(ok = bar_wait(&sh.barD[t], ph.d[t]))) break;
+        ph.d[t] ^= 1u;
+        if (sh.d[t].apply) {
+          const T* co = reinterpret_cast<const T*>(sh.d[t].co);
+          const T cq = co[0], e1 = co[1], e2 = co[2], tau = co[3];
+#pragma unroll
+          for (int j = 0; j < RPT; ++j) {
+            const T d = cq * ql[j] + e1 * d1[j] + e2 * d2[j];
+            d2[j] = d1[j];
+            d1[j] = d;
+            x[j] += tau * d;
+          }
+        }
+        if (sh.d[t].stop) break;
+      }
+      if (!(ok = bar_wait(&sh.barC, ph.c))) break;
+      ph.c ^= 1u;
+      const T* co = reinterpret_cast<const T*>(sh.c);
+      const T c1 = co[0], c2 = co[1], c3 = co[2];
+      acc = T(0);
+#pragma unroll
+      for (int j = 0; j < RPT; ++j) {
+        const T qn = p[j] * mi[j] * c1 - c2 * q[j] - c3 * qm[j];
+        ql[j] = qm[j];
+        qm[j] = q[j];
+        q[j] = qn;
+        acc += m[j] * qn * qn;
+      }
+      publish(acc);
+    }
+    if (!ok) sh.fail = 1;
+    ph.b = pb;
+    if (!run) ph.b ^= 1u;                        // nothing to do: B was not waited for
+    T* xo = reinterpret_cast<T*>(job.x);
+#pragma unroll
+    for (int j = 0; j < RPT; ++j)
+      if (owned(j)) xo[r0 + lrow(j)] = x[j];
+  } else if (wid == -1) {
+    // ---- beta warp
+    double ib = 1.0;                             // 1 / beta_{k-1} (beta_0 = 1)
+    bool ok = true;
+    for (int k = 1;; ++k) {
+      if (!(ok = take(&sh.barB, bytesB, ph.b))) break;
+      const double sum = clu_total(sh.slotB, np);            // beta_k^2
+      const double ibp = ib;
+      ib = sum > 0.0 ? rsqrt(sum) : 0.0;
+      // lane 0: beta_k, then beta_k / beta_{k-1}; lane 1: 1 / (2 beta_k^2), 1 / (2 beta_k^3)
+      const double u = (lane & 1 ? 0.5 * ib : (sum >= 0.0 ? sum : NAN)) * ib;
+      const double w = u * (lane & 1 ? ib : ibp);
+      const int t = k & 1;
+      if (lane < 2) {
+        sh.f[t][lane ? 4 : 1] = u;
+        sh.f[t][lane ? 5 : 6] = w;
+        if (lane == 0) { sh.f[t][0] = sum; sh.f[t][2] = ibp; sh.f[t][3] = ib; }
+      }
+      __syncwarp();
+      if (lane == 0) bar_arrive(&sh.barF[t]);
+      // this iteration's B is the last one once step k - 2 (k = 1: the initial
+      // state) says stop
+      if (k == 1 || k > 2) {
+        const int v = k == 1 ? 0 : t;
+        if (!(ok = bar_wait(&sh.barD[v], ph.d[v]))) break;
+        ph.d[v] ^= 1u;
+        if (sh.d[v].stop) break;
+      }
+    }
+    if (!ok) sh.fail = 1;
+  } else if (wid == -CLU_CW) {
+    // ---- alpha warp (its first sum: the rows with M_ii = 0, handed on as alpha_0)
+    bool ok = true;
+    for (int k = 0;; ++k) {
+      const int t = k & 1;
+      if (!(ok = take(&sh.barA, bytesA, ph.a))) break;
+      if (k > 0) {
+        if (!(ok = bar_wait(&sh.barF[t], ph.f[t]))) break;
+        ph.f[t] ^= 1u;
+      }
+      if (k > 2) {
+        if (!(ok = bar_wait(&sh.barD[t], ph.d[t]))) break;
+        ph.d[t] ^= 1u;
+        if (sh.d[t].stop) break;
+      }
+      const double tot = clu_total(sh.slotA, np);
+      if (k == 0) {
+        if (lane == 0) { sh.alpha[0] = tot; bar_arrive(&sh.barE[0]); }
+        if (!(ok = bar_wait(&sh.barD[0], ph.d[0]))) break;
+        ph.d[0] ^= 1u;
+        if (sh.d[0].stop) {                      // beta_1 came, but no product follows
+          ph.f[1] ^= 1u;
+          break;
+        }
+        continue;
+      }
+      // c2 = alpha_k / beta_k, alpha_k = q.p / beta_k^2 (p doubled)
+      const double al = tot * sh.f[t][lane & 1 ? 4 : 5];
+      if (lane == 0) {
+        T* co = reinterpret_cast<T*>(sh.c);
+        co[0] = (T)sh.f[t][3]; co[1] = (T)al; co[2] = (T)sh.f[t][6];
+        bar_arrive(&sh.barC);
+      }
+      if (lane == 1) { sh.alpha[t] = al; bar_arrive(&sh.barE[t]); }
+    }
+    if (!ok) sh.fail = 1;
+  } else if (wid == 1 - CLU_CW) {
+    // ---- rotation warp: step k - 1 in iteration k (k = 1: the initial state)
+    MinresState S{};
+    bool ok = true;
+    for (int k = 1;; ++k) {
+      const int t = k & 1, u = t ^ 1;
+      if (!(ok = bar_wait(&sh.barF[t], ph.f[t]))) break;
+      ph.f[t] ^= 1u;
+      if (!(ok = bar_wait(&sh.barE[u], ph.e[u]))) break;
+      ph.e[u] ^= 1u;
+      if (S.done != 0) break;                    // an iteration begun past the last step
+      const double al = sh.alpha[u];
+      if (k == 1) {
+        init_state(S, sh.f[t][0], al, job.tol, job.kmax, sigma);
+      } else {
+        S.alpha = al;
+        S.pending = 0;
+        clu_givens(S, sh.f[t][0], sh.f[t][1], sh.f[t][2]);
+      }
+      if (lane == 0) {
+        T* co = reinterpret_cast<T*>(sh.d[u].co);
+        co[0] = (T)S.cq; co[1] = (T)S.cd1; co[2] = (T)S.cd2; co[3] = (T)S.tau;
+        sh.d[u].apply = S.pending;
+        sh.d[u].stop = S.done != 0;
+        bar_arrive(&sh.barD[u]);
+      }
+      if (S.done != 0 && k == 1) break;
+    }
+    if (!ok) { sh.fail = 1; S.status = HS_TIMEOUT; }
+    S.pending = 0;
+    S.done = 2;
+    if (lane == 0) {
+      sh.S = S;
+      if (me == 0 && job.st) *job.st = S;
+    }
+  }
+  __syncthreads();
+  return sh.fail == 0;
+}
+
+}  // namespace hs

@@ -704,6 +704,13 @@ int pipe_replace_period();
 hs_status solve_smem_job(hs_handle* hd, const void* b, const MinresVecs& v, hs_dtype dt, int pc,
                          double tol, long long kmax, bool one);
 
+// minres_clu.cu: the cluster form. clu_choice: CTAs per cluster for n rows on
+// at most sms SMs, 0 where the form does not apply. solve_clu: one solve, x in
+// x and the state in hd->h_state; HS_CUDA without a message when it cannot run.
+int clu_choice(long long n, int sms);
+hs_status solve_clu(hs_handle* hd, const void* b, void* x, hs_dtype dt, int pc, double tol,
+                    long long kmax, int cs);
+
 // Contiguous block ranges per CTA with balanced row counts, cached per grid
 // size (minres.cu).
 hs_status smr_plan(hs_handle* hd, int G, int** d_first, int* rows_cap, int* hdr_cap);
