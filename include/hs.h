@@ -121,8 +121,9 @@ hs_status hs_dim(const hs_handle* hd, long long* n_out);
 hs_status hs_get_sigma(const hs_handle* hd, double* sigma_out);
 hs_status hs_set_sigma(hs_handle* hd, double sigma);
 
-/* Extremal eigenvalues by plain FP64 Lanczos on H (three-term recurrence,
- * T_k re-diagonalised every 10 steps) until both move by < tol; returns
+/* Extremal eigenvalues by plain FP64 Lanczos on H (three-term recurrence)
+ * until both move by < tol over 10 steps (checked every 10 steps; for chains of
+ * up to 4096 rows after 96, 192, ... steps, each run one launch); returns
  * E_min, E_max and (E_min + E_max) / 2 without changing the handle's sigma.
  * Sec. IV A defines sigma from these. */
 hs_status hs_extremal(hs_handle* hd, int max_steps, double tol, double* emin_out,
@@ -214,7 +215,9 @@ hs_status hs_eigs_host(int L, const double* h_host, double sigma, int K, int m_m
  * Algorithm 1 on each on the device (FP64 inner solves by Algorithm 2 with pc,
  * relative tolerance minres_tol, at most 50 n iterations; full
  * reorthogonalisation; the convergence test on T_k); m (m_max, else
- * max(130, 3K + 30)) is at most 256. The group size per (L, pc, SM count) is
+ * max(130, 3K + 30)) is at most 256. Where every chain has at most 4096 rows
+ * the groups are thread-block clusters and share one queue, the longest chains
+ * first. The group size per (L, pc, SM count) is
  * timed on first use and cached in the JSON file HS_SWEEP_TUNE (default
  * $HOME/.cache/hs_sweep_tune.json); HS_SWEEP_S forces it.
  * Outputs (host, realisation r at offset r K): evals_host (B K, each ordered as

@@ -45,4 +45,8 @@ hs_status lz_step(LzRun& r, hs_status solve_status, long long iters, int sweeps)
 hs_status lz_finish(LzRun& r, double* evals_host, double* evecs_dev, double* resid_host,
                     hs_lanczos_info* info);
 
+// sigma = (E_min + E_max) / 2 for each handle (all on one stream and device):
+// hs_extremal's values, for short chains in one launch per chain length.
+hs_status midpoints(const std::vector<hs_handle*>& hds);
+
 }  // namespace hs

@@ -716,7 +716,7 @@ static bool pipe_choice(const hs_handle* hd, bool f64, int pc) {
 static int cluster_choice(const hs_handle* hd, bool f64, int pc) {
   if (getenv("HS_MINRES_PIPE") || getenv("HS_BARRIER_LIMIT")) return 0;
   // FP64 above 4096 rows: 16 SMs' FP64 pipes would bound it
-  if (f64 && hd->n > 4096 && pipe_choice(hd, f64, pc)) return 0;
+  if (f64 && hd->n > CLU_F64_ROWS && pipe_choice(hd, f64, pc)) return 0;
   const int bud = hd->sm_budget.load(std::memory_order_relaxed);
   return clu_choice(hd->n, std::max(1, std::min(hd->num_sms, bud > 0 ? bud : hd->num_sms)));
 }

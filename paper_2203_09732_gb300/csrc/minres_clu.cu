@@ -20,48 +20,45 @@ __global__ void __launch_bounds__(CLU_NT, 1) k_minres_clu(SmemJob job, int pc) {
   clu_sync();   // no CTA leaves while another may still write to it
 }
 
+// One FP64 solve per cluster: jobs[blockIdx.x / cs] (all of one L), the
+// Lanczos scalars in trace + cluster * tstride where trace is set.
+__global__ void __launch_bounds__(CLU_NT, 1) k_minres_clu_many(const SmemJob* jobs, int pc,
+                                                               double* trace, long long tstride) {
+  extern __shared__ __align__(16) char dyn[];
+  __shared__ CluShared sh;
+  __shared__ SmemJob sj;
+  clu_setup(sh);
+  CluPhase ph;
+  const int cs = (int)clu_size(), id = (int)blockIdx.x / cs;
+  if (threadIdx.x == 0) sj = jobs[id];
+  __syncthreads();
+  clu_solve64(clu_rpt((int)sj.g.n, cs), sj, pc, sh, dyn, ph, trace ? trace + id * tstride : nullptr);
+  clu_sync();
+}
+
 template <typename T, int RPT>
 hs_status launch_t(hs_handle* hd, const SmemJob& job, int pc, int cs) {
-  const size_t sm = clu_bytes<T>((int)hd->n, hd->L, cs, RPT);
-  auto kern = k_minres_clu<T, RPT>;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(cs);
-  cfg.blockDim = dim3(CLU_NT);
-  cfg.dynamicSmemBytes = sm;
-  cfg.stream = hd->stream;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = cs;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) !=
-          cudaSuccess ||
-      (cs > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
-                     cudaSuccess) ||
-      cudaLaunchKernelEx(&cfg, kern, job, pc) != cudaSuccess) {
-    cudaGetLastError();
-    return HS_CUDA;
-  }
-  count_launches(1);
-  return HS_OK;
+  return clu_launch(k_minres_clu<T, RPT>, cs, cs, clu_bytes<T>((int)hd->n, hd->L, cs, RPT),
+                    hd->stream, job, pc)
+             ? HS_OK : HS_CUDA;
 }
 
 template <typename T>
 hs_status launch_rpt(hs_handle* hd, const SmemJob& job, int pc, int cs) {
-  const int rpc = ((int)hd->n + cs - 1) / cs;
-  const int rpt = (rpc + 32 * CLU_NW - 1) / (32 * CLU_NW);
+  const int rpt = clu_rpt((int)hd->n, cs);
   // rows per thread: as few as hold the rows in FP64 (each row is FP64 work on
   // the critical path); two at least in FP32, where half the warps make half
   // the partials and messages (n = 924, 8 CTAs: 1.72 -> 1.59 us per iteration;
   // FP64 there 2.38 -> 3.00)
   if constexpr (sizeof(T) == 8)
-    if (rpt <= 1) return launch_t<T, 1>(hd, job, pc, cs);
-  if (rpt <= 2) return launch_t<T, 2>(hd, job, pc, cs);
-  if (rpt <= 4) return launch_t<T, 4>(hd, job, pc, cs);
-  if (rpt <= CLU_RPT_MAX) return launch_t<T, CLU_RPT_MAX>(hd, job, pc, cs);
-  return HS_CUDA;
+    if (rpt == 1) return launch_t<T, 1>(hd, job, pc, cs);
+  switch (rpt) {
+    case 1:
+    case 2: return launch_t<T, 2>(hd, job, pc, cs);
+    case 4: return launch_t<T, 4>(hd, job, pc, cs);
+    case CLU_RPT_MAX: return launch_t<T, CLU_RPT_MAX>(hd, job, pc, cs);
+    default: return HS_CUDA;
+  }
 }
 
 }  // namespace
@@ -94,6 +91,15 @@ hs_status solve_clu(hs_handle* hd, const void* b, void* x, hs_dtype dt, int pc, 
                                   cudaMemcpyDeviceToHost, hd->stream));
   HS_CUDA_TRY(hd, cudaStreamSynchronize(hd->stream));
   return HS_OK;
+}
+
+hs_status launch_clu_many(const SmemJob* jobs, int count, int n, int L, int pc, int cs,
+                          cudaStream_t s, double* trace, long long tstride) {
+  const int rpt = clu_rpt(n, cs);
+  if (!rpt) return HS_CUDA;
+  return clu_launch(k_minres_clu_many, count * cs, cs, clu_bytes<double>(n, L, cs, rpt), s, jobs, pc,
+                    trace, tstride)
+             ? HS_OK : HS_CUDA;
 }
 
 }  // namespace hs

@@ -226,7 +226,9 @@ __device__ __forceinline__ void clu_givens(MinresState& S, double sumsq, double 
 }
 
 // One solve by one cluster; every thread of every CTA calls it with the same
-// job. Rows are dealt to the CTAs in contiguous runs of rank order. Returns
+// job. Where trace is set, CTA 0 writes alpha_k to trace[2 (k - 1)] and beta_{k+1}
+// to trace[2 (k - 1) + 1] (k = 1 .. kmax): the tridiagonal matrix of the Lanczos
+// process that MINRES runs on. Rows are dealt to the CTAs in contiguous runs of rank order. Returns
 // false when a wait gave up (status HS_TIMEOUT). The final state is in sh.S of
 // every CTA and, if job.st is set, in *job.st.
 //
@@ -242,7 +244,8 @@ __device__ __forceinline__ void clu_givens(MinresState& S, double sumsq, double 
 //   rotation  wait F (beta_k) and E (alpha_{k-1}): the rotation of step k - 1; D: its
 //             coefficients
 template <typename T, int RPT>
-__device__ bool clu_solve(const SmemJob& job, int pc, CluShared& sh, char* dyn, CluPhase& ph) {
+__device__ bool clu_solve(const SmemJob& job, int pc, CluShared& sh, char* dyn, CluPhase& ph,
+                          double* trace = nullptr) {
   const Geo& g = job.g;
   const int n = (int)g.n;
   const int cs = (int)clu_size(), me = (int)clu_rank();
@@ -425,10 +428,10 @@ __device__ bool clu_solve(const SmemJob& job, int pc, CluShared& sh, char* dyn, 
     if (!ok) sh.fail = 1;
     ph.b = pb;
     if (!run) ph.b ^= 1u;                        // nothing to do: B was not waited for
-    T* xo = reinterpret_cast<T*>(job.x);
+    T* xo = reinterpret_cast<T*>(job.x);         // may be null (trace runs)
 #pragma unroll
     for (int j = 0; j < RPT; ++j)
-      if (owned(j)) xo[r0 + lrow(j)] = x[j];
+      if (xo && owned(j)) xo[r0 + lrow(j)] = x[j];
   } else if (wid == -1) {
     // ---- beta warp
     double ib = 1.0;                             // 1 / beta_{k-1} (beta_0 = 1)
@@ -447,6 +450,7 @@ __device__ bool clu_solve(const SmemJob& job, int pc, CluShared& sh, char* dyn, 
         sh.f[t][lane ? 5 : 6] = w;
         if (lane == 0) { sh.f[t][0] = sum; sh.f[t][2] = ibp; sh.f[t][3] = ib; }
       }
+      if (trace && me == 0 && lane == 0 && k > 1 && k - 1 <= job.kmax) trace[2 * (k - 2) + 1] = u;
       __syncwarp();
       if (lane == 0) bar_arrive(&sh.barF[t]);
       // this iteration's B is the last one once step k - 2 (k = 1: the initial
@@ -493,6 +497,7 @@ __device__ bool clu_solve(const SmemJob& job, int pc, CluShared& sh, char* dyn, 
         bar_arrive(&sh.barC);
       }
       if (lane == 1) { sh.alpha[t] = al; bar_arrive(&sh.barE[t]); }
+      if (trace && me == 0 && lane == 1 && k <= job.kmax) trace[2 * (k - 1)] = al;
     }
     if (!ok) sh.fail = 1;
   } else if (wid == 1 - CLU_CW) {
@@ -533,6 +538,51 @@ __device__ bool clu_solve(const SmemJob& job, int pc, CluShared& sh, char* dyn, 
   }
   __syncthreads();
   return sh.fail == 0;
+}
+
+// The rows per thread that a chain of n rows needs on cs CTAs; 0: too many.
+__host__ __device__ inline int clu_rpt(int n, int cs) {
+  const int need = ((n + cs - 1) / cs + 32 * CLU_NW - 1) / (32 * CLU_NW);
+  return need <= 1 ? 1 : need <= 2 ? 2 : need <= 4 ? 4 : need <= CLU_RPT_MAX ? CLU_RPT_MAX : 0;
+}
+
+// clu_solve in FP64 with the rows per thread chosen at run time.
+__device__ inline bool clu_solve64(int rpt, const SmemJob& job, int pc, CluShared& sh, char* dyn,
+                                   CluPhase& ph, double* trace = nullptr) {
+  switch (rpt) {
+    case 1: return clu_solve<double, 1>(job, pc, sh, dyn, ph, trace);
+    case 2: return clu_solve<double, 2>(job, pc, sh, dyn, ph, trace);
+    case 4: return clu_solve<double, 4>(job, pc, sh, dyn, ph, trace);
+    default: return clu_solve<double, CLU_RPT_MAX>(job, pc, sh, dyn, ph, trace);
+  }
+}
+
+// Launch of a kernel on clusters of cs CTAs (grid: a multiple of cs); false
+// when it is refused.
+template <typename K, typename... A>
+inline bool clu_launch(K kern, int grid, int cs, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(CLU_NT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cs;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+          cudaSuccess ||
+      (cs > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+                     cudaSuccess) ||
+      cudaLaunchKernelEx(&cfg, kern, args...) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  count_launches(1);
+  return true;
 }
 
 }  // namespace hs

@@ -710,6 +710,13 @@ hs_status solve_smem_job(hs_handle* hd, const void* b, const MinresVecs& v, hs_d
 int clu_choice(long long n, int sms);
 hs_status solve_clu(hs_handle* hd, const void* b, void* x, hs_dtype dt, int pc, double tol,
                     long long kmax, int cs);
+// FP64 solves of one chain length, one per cluster: jobs[0..count) (device);
+// trace (device, may be null): the alpha_k, beta_{k+1} of job j at trace +
+// j tstride. Asynchronous.
+hs_status launch_clu_many(const SmemJob* jobs, int count, int n, int L, int pc, int cs,
+                          cudaStream_t s, double* trace, long long tstride);
+// FP64 solves of at most this many rows run in a cluster.
+constexpr long long CLU_F64_ROWS = 4096;
 
 // Contiguous block ranges per CTA with balanced row counts, cached per grid
 // size (minres.cu).

@@ -22,7 +22,7 @@
 #include <sys/stat.h>
 
 #include "lanczos.cuh"
-#include "minres_smem.cuh"
+#include "minres_clu.cuh"
 
 namespace hs {
 
@@ -305,6 +305,7 @@ struct SweepReal {
   MinresState* st;        // state of the last inner solve
   int* res;               // [0] steps, [1] converged pairs, [2] status, [3] unconverged solves
   long long* iters;       // MINRES iterations of all its solves
+  int m;                  // Lanczos step cap
 };
 
 // The device form's arguments of one queue: its realisations, queue head
@@ -390,7 +391,11 @@ __device__ int ritz_converged(int kk, const double* alpha, const double* beta, d
       for (int i = m - 1; i >= l; --i) {
         const double f = s * e[i];
         const double b = cc * e[i];
-        r = hypot(f, g);
+        // one reciprocal root for r, f / r and g / r (7 FP64 instructions; a
+        // hypot and two divisions are about 35, at 64 cycles each)
+        const double rr = f * f + g * g;
+        const double ir = rr > 0.0 ? rsqrt(rr) : 0.0;
+        r = rr * ir;
         e[i + 1] = r;
         if (r == 0.0) {
           d[i + 1] -= p;
@@ -398,8 +403,8 @@ __device__ int ritz_converged(int kk, const double* alpha, const double* beta, d
           underflow = true;
           break;
         }
-        s = f / r;
-        cc = g / r;
+        s = f * ir;
+        cc = g * ir;
         g = d[i + 1] - p;
         r = (d[i] - g) * s + 2.0 * cc * b;
         p = s * r;
@@ -573,6 +578,259 @@ __global__ void __launch_bounds__(NT, 1) k_sweep(SweepArgs a0, SmemQueue q0, Swe
   }
 }
 
+// ---------------------------------------------------------------------------
+// Cluster form, for chains of up to CLU_F64_ROWS rows: a thread-block cluster
+// takes a realisation (longest chains first) and runs all of Algorithm 1 on it,
+// the inner solves by clu_solve. 24 chains of L = 10 and 8 of L = 12, 4 pairs
+// each, all calls included: 1063 -> 139 ms (the launch 1009 -> 131 ms: groups of
+// one CTA were bound by one SM's FP64 pipe, larger ones by the exchange through
+// L2; the setup 126 -> 7 ms: sigma of all chains of a length in one launch).
+constexpr int CSW_NW = CLU_NT / 32;
+
+struct CluSweepShared {
+  CluShared clu;
+  SmemJob job;
+  SweepReal r;
+  int rid;
+  double sum[2][CLU_SIZE_MAX];       // CTA sums, in turn
+  double warp[CSW_NW][8];
+  double part[VRED], hcoef[VRED];
+  double alpha[SWEEP_MMAX], beta[SWEEP_MMAX];
+  double qd[SWEEP_MMAX], qe[SWEEP_MMAX], qz[SWEEP_MMAX];
+  int flag[2];
+};
+
+// Sum of one value per thread over the cluster, the same in every thread.
+// turn alternates the places of the CTA sums, so that one cluster barrier is
+// enough: a place is written again only after the barrier of the next sum.
+__device__ __forceinline__ double clu_sum(CluSweepShared& sh, double v, int& turn) {
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int cs = (int)clu_size(), me = (int)clu_rank();
+  v = warp_sum_all(v);
+  if (lane == 0) sh.warp[wid][0] = v;
+  __syncthreads();
+  if ((int)threadIdx.x < cs) {
+    double t = 0.0;
+    for (int w = 0; w < CSW_NW; ++w) t += sh.warp[w][0];
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(
+                     clu_map(smem_u32(&sh.sum[turn][me]), threadIdx.x)), "d"(t) : "memory");
+  }
+  clu_sync();
+  double t = 0.0;
+  for (int c = 0; c < cs; ++c) t += sh.sum[turn][c];
+  turn ^= 1;
+  return t;
+}
+
+__global__ void __launch_bounds__(CLU_NT, 1) k_sweep_clu(const SweepReal* reals, int count, int* head,
+                                                         int K, double tol, double minres_tol,
+                                                         int pc) {
+  extern __shared__ __align__(16) char dyn[];
+  __shared__ CluSweepShared sh;
+  clu_setup(sh.clu);
+  CluPhase ph;
+  const int cs = (int)clu_size(), me = (int)clu_rank();
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int NT = CLU_NT;
+  int turn = 0;
+  while (true) {
+    if (me == 0 && threadIdx.x == 0) {
+      const int id = atomicAdd(head, 1);
+      for (int c = 0; c < cs; ++c)
+        asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(clu_map(smem_u32(&sh.rid), c)),
+                     "r"(id) : "memory");
+    }
+    clu_sync();
+    const int rid = sh.rid;
+    if (rid >= count) break;
+    if (threadIdx.x == 0) sh.r = reals[rid];
+    __syncthreads();
+    const SweepReal& sr = sh.r;
+    const long long n = sr.g.n;
+    const int rpt = clu_rpt((int)n, cs), rpc = clu_rows((int)n, cs, rpt);
+    const long long lo = min(n, (long long)me * rpc), hi = min(n, lo + rpc);   // this CTA's rows
+    int k = 0, unconv = 0, status = HS_OK;
+    long long iters = 0;
+    double bk = 0.0;
+    bool done = false, skip = false;
+    while (!done) {
+      const double* vk = sr.V + (size_t)k * n;
+      // (H - sigma) x = v_k
+      if (threadIdx.x == 0)
+        sh.job = SmemJob{sr.g, vk, sr.x, nullptr, sr.sigma, minres_tol, 50 * n};
+      __syncthreads();
+      const bool ok = clu_solve64(rpt, sh.job, pc, sh.clu, dyn, ph);
+      const MinresState& S = sh.clu.S;
+      if (!ok || S.status != HS_OK) { status = ok ? S.status : HS_TIMEOUT; break; }
+      iters += S.k - 1;
+      if (S.beta1 > 0 && !(fabs(S.phi) < S.tol_abs) && S.beta != 0.0) ++unconv;
+      // w = x - beta_k v_{k-1}; alpha_k = v_k . w; w -= alpha_k v_k
+      const double* vkm = k > 0 ? sr.V + (size_t)(k - 1) * n : nullptr;
+      double pa = 0.0;
+      for (long long i = lo + threadIdx.x; i < hi; i += NT) {
+        const double wi = sr.x[i] - (k > 0 ? bk * vkm[i] : 0.0);
+        sr.w[i] = wi;
+        pa += vk[i] * wi;
+      }
+      const double al = clu_sum(sh, pa, turn);
+      for (long long i = lo + threadIdx.x; i < hi; i += NT) sr.w[i] -= al * vk[i];
+      // full reorthogonalisation against v_1..v_k: two classical Gram-Schmidt passes
+      for (int pass = 0; pass < 2; ++pass) {
+        for (int j0 = 0; j0 <= k; j0 += 8) {
+          double acc[8];
+#pragma unroll
+          for (int jj = 0; jj < 8; ++jj) acc[jj] = 0.0;
+          for (long long i = lo + threadIdx.x; i < hi; i += NT) {
+            const double wi = sr.w[i];
+#pragma unroll
+            for (int jj = 0; jj < 8; ++jj)
+              if (j0 + jj <= k) acc[jj] += sr.V[(size_t)(j0 + jj) * n + i] * wi;
+          }
+#pragma unroll
+          for (int jj = 0; jj < 8; ++jj)
+            if (j0 + jj <= k) {
+              const double t = warp_sum_all(acc[jj]);
+              if (lane == 0) sh.warp[wid][jj] = t;
+            }
+          __syncthreads();
+          if (threadIdx.x < 8 && j0 + (int)threadIdx.x <= k) {
+            double t = 0.0;
+            for (int w = 0; w < CSW_NW; ++w) t += sh.warp[w][threadIdx.x];
+            sh.part[j0 + threadIdx.x] = t;
+          }
+          __syncthreads();
+        }
+        clu_sync();                              // every CTA's part[] is written
+        for (int j = threadIdx.x; j <= k; j += NT) {
+          double t = 0.0;
+          for (int c = 0; c < cs; ++c) {
+            double v;
+            asm volatile("ld.shared::cluster.f64 %0, [%1];"
+                         : "=d"(v) : "r"(clu_map(smem_u32(&sh.part[j]), c)) : "memory");
+            t += v;
+          }
+          sh.hcoef[j] = t;
+        }
+        clu_sync();                              // and read
+        for (long long i = lo + threadIdx.x; i < hi; i += NT) {
+          double wi = sr.w[i];
+          for (int j = 0; j <= k; ++j) wi -= sh.hcoef[j] * sr.V[(size_t)j * n + i];
+          sr.w[i] = wi;
+        }
+      }
+      double pb = 0.0;
+      for (long long i = lo + threadIdx.x; i < hi; i += NT) pb += sr.w[i] * sr.w[i];
+      const double bn = sqrt(fmax(clu_sum(sh, pb, turn), 0.0));
+      // the convergence test (every CTA's thread 0 on the same numbers). It takes
+      // about as long as 0.3 kk^2 iterations of a solve, so the step after one that
+      // left two pairs or more open goes without
+      if (threadIdx.x == 0) {
+        sh.alpha[k] = al;
+        const int kk = k + 1;
+        const bool last = bn <= 1e-13 * fabs(al) || kk == sr.m;
+        int nconv = 0;
+        if (kk >= K && (last || !skip)) {
+          nconv = ritz_converged(kk, sh.alpha, sh.beta, bn, K, tol, sh.qd, sh.qe, sh.qz);
+          skip = nconv < K - 1;
+        } else {
+          skip = false;
+        }
+        const bool stop = nconv == K || last;
+        sh.flag[0] = stop ? 1 : 0;
+        sh.flag[1] = nconv;
+        if (!stop) sh.beta[k] = bn;
+      }
+      __syncthreads();
+      done = sh.flag[0] != 0;
+      if (!done) {
+        double* vn = sr.V + (size_t)(k + 1) * n;
+        const double ib = 1.0 / bn;
+        for (long long i = lo + threadIdx.x; i < hi; i += NT) vn[i] = sr.w[i] * ib;
+        bk = bn;
+        ++k;
+      }
+      __syncthreads();
+    }
+    if (me == 0 && threadIdx.x == 0) {
+      const int steps = status == HS_OK ? k + 1 : k;
+      for (int j = 0; j < steps; ++j) sr.alpha[j] = sh.alpha[j];
+      for (int j = 0; j + 1 < steps; ++j) sr.beta[j] = sh.beta[j];
+      sr.res[0] = steps;
+      sr.res[1] = status == HS_OK ? sh.flag[1] : 0;
+      sr.res[2] = status;
+      sr.res[3] = unconv;
+      *sr.iters = iters;
+    }
+    __syncthreads();
+    if (status == HS_TIMEOUT) break;             // the barriers are out of step
+  }
+  clu_sync();
+}
+
+// Microseconds per FP64 iteration of n rows on a cluster of cs CTAs: the
+// exchanges and reductions, the rows of a thread, the traffic of q (fitted to
+// the measurements at clu_choice, within 15 %).
+double clu_iter_us(long long n, int cs) { return 1.5 + 0.8 * clu_rpt((int)n, cs) + 2.5e-4 * n; }
+
+// The cluster size for a sweep, at least smin: the one whose clusters finish a
+// list of realisations (longest first, each to the cluster that is free first)
+// soonest by clu_iter_us. Work per realisation: about n^1.05 iterations a solve.
+int clu_sweep_size(const std::vector<long long>& ns, int num_sms, int smin) {
+  int best = 0;
+  double best_t = 1e300;
+  for (int cs = 1; cs <= CLU_SIZE_MAX && cs <= num_sms; cs *= 2) {
+    if (cs < smin || !clu_rpt((int)ns[0], cs)) continue;
+    std::vector<double> busy(std::max(1, num_sms / cs), 0.0);
+    for (long long n : ns) {
+      auto it = std::min_element(busy.begin(), busy.end());
+      *it += std::pow((double)n, 1.05) * clu_iter_us(n, cs);
+    }
+    const double t = *std::max_element(busy.begin(), busy.end());
+    if (t < best_t) { best_t = t; best = cs; }
+  }
+  return best;
+}
+
+// The smallest cluster size with the highest throughput on the whole GPU for
+// chains like run r's (clusters x iterations per second of one); 0: none runs.
+hs_status tune_clu(const LzRun& r, int pc, int num_sms, cudaStream_t s, Tune* out) {
+  const int iters = 200;
+  hs_handle* hd = r.hd;
+  SmemJob* jobs = nullptr;
+  hs_status st = dev_alloc(hd, (void**)&jobs, sizeof(SmemJob) * num_sms);
+  if (st != HS_OK) return st;
+  const std::vector<SmemJob> h(num_sms, job_for(hd, r.rhs(), nullptr, nullptr, 0.0, iters));
+  cudaEvent_t e0, e1;
+  cudaEventCreate(&e0);
+  cudaEventCreate(&e1);
+  double best = 0.0;
+  // pageable source: staged before the call returns
+  if (cudaMemcpyAsync(jobs, h.data(), sizeof(SmemJob) * num_sms, cudaMemcpyHostToDevice, s) ==
+      cudaSuccess)
+    for (int cs = 1; cs <= CLU_SIZE_MAX && cs <= num_sms; cs *= 2) {
+      const int groups = num_sms / cs;
+      float ms = 0.f;
+      for (int rep = 0; rep < 2; ++rep) {        // the first one loads the kernel
+        cudaEventRecord(e0, s);
+        if (launch_clu_many(jobs, groups, (int)hd->n, hd->L, pc, cs, s, nullptr, 0) != HS_OK) break;
+        cudaEventRecord(e1, s);
+        if (cudaStreamSynchronize(s) != cudaSuccess) break;
+        cudaEventElapsedTime(&ms, e0, e1);
+      }
+      const double rate = ms > 0 ? iters / (ms * 1e-3) : 0.0;
+      if (rate * groups > best * 1.02) {
+        best = rate * groups;
+        out->S = cs;
+        out->rate = rate;
+      }
+    }
+  cudaGetLastError();
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  dev_free(hd, jobs);
+  return HS_OK;
+}
+
 // Launch of the device form for one or two queues (two-reduction solves,
 // FP64); HS_CUDA when it does not fit or the cooperative launch is refused.
 template <int PC, int JM, int NT>
@@ -699,8 +957,10 @@ extern "C" hs_status hs_sweep(int B, const int* L_host, const double* h_host, in
   int device = 0, num_sms = 0;
   cudaGetDevice(&device);
   cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, device);
+  char* cmem = nullptr;              // the cluster form's records and results
   auto cleanup = [&](hs_status out) {
     cudaStreamSynchronize(s);
+    if (cmem) dev_free(hd[0], cmem);
     for (int c = 0; c < ncls; ++c) {
       free_class(cls[c]);
       cudaFree(dv[c].reals); cudaFree(dv[c].ab); cudaFree(dv[c].res); cudaFree(dv[c].iters);
@@ -718,9 +978,12 @@ extern "C" hs_status hs_sweep(int B, const int* L_host, const double* h_host, in
   {
     size_t off = 0;
     for (int r = 0; r < B; ++r) {
-      st = hs_create(L_host[r], h_host + off, NAN, s, &hd[r]);
+      st = hs_create(L_host[r], h_host + off, 0.0, s, &hd[r]);
       off += L_host[r];
       if (st != HS_OK) return cleanup(st);
+    }
+    if ((st = midpoints(hd)) != HS_OK) return cleanup(st);
+    for (int r = 0; r < B; ++r) {
       if ((st = lz_start(runs[r], hd[r], K, m_max, tol, seed + (unsigned long long)r, nullptr)) !=
           HS_OK)
         return cleanup(st);
@@ -728,6 +991,11 @@ extern "C" hs_status hs_sweep(int B, const int* L_host, const double* h_host, in
     }
   }
   if (cudaMalloc(&err, sizeof(int)) != cudaSuccess) return cleanup(HS_OOM);
+  if (cudaMemsetAsync(err, 0, sizeof(int), s) != cudaSuccess) return cleanup(HS_CUDA);
+  // short chains: one cluster per realisation at a time
+  bool clu = !getenv("HS_SWEEP_S");
+  for (int r = 0; r < B; ++r)
+    clu = clu && hd[r]->n <= CLU_F64_ROWS && clu_choice(hd[r]->n, num_sms) > 0;
   // group size per class: forced (HS_SWEEP_S), cached or timed
   auto tunes = tune_read();
   bool tunes_changed = false;
@@ -735,9 +1003,9 @@ extern "C" hs_status hs_sweep(int B, const int* L_host, const double* h_host, in
     Class& C = cls[c];
     C.hd0 = hd[C.idx[0]];
     C.n = C.hd0->n;
-    if ((st = alloc_class(C, num_sms)) != HS_OK) return cleanup(st);
+    if (!clu && (st = alloc_class(C, num_sms)) != HS_OK) return cleanup(st);
     char key[96];
-    snprintf(key, sizeof key, "L%d_pc%d_f64_sm%d", C.L, (int)pc, num_sms);
+    snprintf(key, sizeof key, "L%d_pc%d_f64_%ssm%d", C.L, (int)pc, clu ? "clu_" : "", num_sms);
     if (const char* fs = getenv("HS_SWEEP_S")) {
       C.tune.S = std::max(1, std::min(num_sms, atoi(fs)));
       C.tune.rate = 1.0;
@@ -746,7 +1014,11 @@ extern "C" hs_status hs_sweep(int B, const int* L_host, const double* h_host, in
       C.tune = tunes[key];
       C.tuned = 0;
     } else {
-      if ((st = tune_class(C, runs, pc, num_sms, device, s, err, 0)) != HS_OK) return cleanup(st);
+      st = clu ? tune_clu(runs[C.idx[0]], pc, num_sms, s, &C.tune)
+               : tune_class(C, runs, pc, num_sms, device, s, err, 0);
+      if (st == HS_OK && !C.tune.S) st = HS_CUDA;
+      if (st != HS_OK) return cleanup(st);
+      C.tuned = 1;
       tunes[key] = C.tune;
       tunes_changed = true;
     }
@@ -762,6 +1034,7 @@ extern "C" hs_status hs_sweep(int B, const int* L_host, const double* h_host, in
     Class& C = cls[c];
     Dev& D = dv[c];
     const int nr = (int)C.idx.size();
+    if (clu) continue;
     if (cudaMalloc(&D.reals, sizeof(SweepReal) * nr) != cudaSuccess ||
         cudaMalloc(&D.ab, sizeof(double) * 2 * SWEEP_MMAX * nr) != cudaSuccess ||
         cudaMalloc(&D.res, sizeof(int) * 4 * nr) != cudaSuccess ||
@@ -785,6 +1058,7 @@ extern "C" hs_status hs_sweep(int B, const int* L_host, const double* h_host, in
       R.st = C.states + j;
       R.res = D.res + 4 * j;
       R.iters = D.iters + j;
+      R.m = runs[r].m;
     }
     C.h_head[0] = 0;
     C.h_head[1] = nr;
@@ -798,13 +1072,61 @@ extern "C" hs_status hs_sweep(int B, const int* L_host, const double* h_host, in
       return cleanup(HS_CUDA);
     }
   }
+  // the cluster form: one list of all realisations, the longest chains first
+  std::vector<int> list(B);
+  const size_t ab_bytes = sizeof(double) * 2 * SWEEP_MMAX * B, it_bytes = sizeof(long long) * B,
+               res_bytes = sizeof(int) * 4 * B, re_bytes = (sizeof(SweepReal) * B + 15) & ~size_t(15);
+  int* chead = nullptr;
+  if (clu) {
+    for (int r = 0; r < B; ++r) list[r] = r;
+    std::stable_sort(list.begin(), list.end(), [&](int a, int b) { return hd[a]->n > hd[b]->n; });
+    if ((st = dev_alloc(hd[0], (void**)&cmem, ab_bytes + it_bytes + res_bytes + re_bytes + 16)) !=
+        HS_OK)
+      return cleanup(st);
+    double* ab = reinterpret_cast<double*>(cmem);
+    long long* its = reinterpret_cast<long long*>(cmem + ab_bytes);
+    int* res = reinterpret_cast<int*>(cmem + ab_bytes + it_bytes);
+    chead = reinterpret_cast<int*>(cmem + ab_bytes + it_bytes + res_bytes);
+    std::vector<SweepReal> hr(B);
+    for (int j = 0; j < B; ++j) {
+      const int r = list[j];
+      hr[j] = SweepReal{hd[r]->geo(), hd[r]->sigma, runs[r].V, runs[r].x, runs[r].w,
+                        ab + (size_t)2 * SWEEP_MMAX * j, ab + (size_t)2 * SWEEP_MMAX * j + SWEEP_MMAX,
+                        nullptr, res + 4 * j, its + j, runs[r].m};
+    }
+    if (cudaMemsetAsync(cmem + ab_bytes, 0, it_bytes + res_bytes + 16, s) != cudaSuccess ||
+        cudaMemcpyAsync(cmem + ab_bytes + it_bytes + res_bytes + 16, hr.data(),
+                        sizeof(SweepReal) * B, cudaMemcpyHostToDevice, s) != cudaSuccess) {
+      cudaGetLastError();
+      return cleanup(HS_CUDA);
+    }
+  }
   const double t_setup = std::chrono::duration<double>(clk::now() - t0).count();
   // the launch: groups per class from the split of the SMs; a group size that
   // does not fit the kernel's shared memory grows by one CTA until it fits
   const auto ts = clk::now();
   const unsigned long long limit = 1ull << 22;
   hs_status ls = HS_CUDA;
-  for (int attempt = 0; attempt < 64 && ls == HS_CUDA; ++attempt) {
+  if (clu) {
+    std::vector<long long> ns(B);
+    for (int j = 0; j < B; ++j) ns[j] = hd[list[j]]->n;
+    int smin = 1;
+    for (int c = 0; c < ncls; ++c) smin = std::max(smin, cls[c].tune.S);
+    const int cs = clu_sweep_size(ns, num_sms, std::min(smin, num_sms));
+    const int groups = cs > 0 ? std::min(B, num_sms / cs) : 0;
+    size_t sm = 0;
+    for (int c = 0; c < ncls && cs > 0; ++c) {
+      sm = std::max(sm, clu_bytes<double>((int)cls[c].n, cls[c].L, cs, clu_rpt((int)cls[c].n, cs)));
+      cls[c].tune.S = cs;
+      cls[c].ngroups = groups;
+    }
+    if (cs > 0 &&
+        clu_launch(k_sweep_clu, groups * cs, cs, sm, s,
+                   reinterpret_cast<const SweepReal*>(cmem + ab_bytes + it_bytes + res_bytes + 16), B,
+                   chead, K, tol, minres_tol, (int)pc))
+      ls = HS_OK;
+  }
+  for (int attempt = 0; !clu && attempt < 64 && ls == HS_CUDA; ++attempt) {
     split_groups(cls, ncls, num_sms);
     int used = 0;
     for (int c = 0; c < ncls; ++c) {
@@ -849,26 +1171,32 @@ extern "C" hs_status hs_sweep(int B, const int* L_host, const double* h_host, in
   long long total_iters = 0;
   int max_steps = 0;
   hs_status first_err = HS_OK;
-  for (int c = 0; c < ncls; ++c) {
-    Class& C = cls[c];
-    const int nr = (int)C.idx.size();
+  // one block of results per class, or one of all (the cluster form)
+  for (int c = 0; c < (clu ? 1 : ncls); ++c) {
+    const std::vector<int>& idx = clu ? list : cls[c].idx;
+    const int nr = (int)idx.size();
     std::vector<double> ab((size_t)2 * SWEEP_MMAX * nr);
     std::vector<int> res(4 * (size_t)nr);
     std::vector<long long> its(nr);
-    if (cudaMemcpy(ab.data(), dv[c].ab, sizeof(double) * ab.size(), cudaMemcpyDeviceToHost) !=
+    const void* dab = clu ? (const void*)cmem : dv[c].ab;
+    const void* dits = clu ? (const void*)(cmem + ab_bytes) : dv[c].iters;
+    const void* dres = clu ? (const void*)(cmem + ab_bytes + it_bytes) : dv[c].res;
+    int timeout = 0;
+    if (cudaMemcpyAsync(ab.data(), dab, sizeof(double) * ab.size(), cudaMemcpyDeviceToHost, s) !=
             cudaSuccess ||
-        cudaMemcpy(res.data(), dv[c].res, sizeof(int) * res.size(), cudaMemcpyDeviceToHost) !=
+        cudaMemcpyAsync(res.data(), dres, sizeof(int) * res.size(), cudaMemcpyDeviceToHost, s) !=
             cudaSuccess ||
-        cudaMemcpy(its.data(), dv[c].iters, sizeof(long long) * nr, cudaMemcpyDeviceToHost) !=
-            cudaSuccess) {
+        cudaMemcpyAsync(its.data(), dits, sizeof(long long) * nr, cudaMemcpyDeviceToHost, s) !=
+            cudaSuccess ||
+        cudaMemcpyAsync(&timeout, err, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess) {
       cudaGetLastError();
       return cleanup(HS_CUDA);
     }
-    int timeout = 0;
-    cudaMemcpy(&timeout, err, sizeof(int), cudaMemcpyDeviceToHost);
+    for (int j = 0; clu && j < nr; ++j) timeout |= res[4 * j + 2] == HS_TIMEOUT;
     if (timeout) return cleanup(fail(hd[0], HS_TIMEOUT, "hs_sweep: a group's wait gave up"));
     for (int j = 0; j < nr; ++j) {
-      LzRun& R = runs[C.idx[j]];
+      LzRun& R = runs[idx[j]];
       const int steps = res[4 * j];
       const double* al = &ab[(size_t)2 * SWEEP_MMAX * j];
       R.alpha.assign(al, al + steps);
