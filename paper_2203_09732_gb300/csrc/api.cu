@@ -371,6 +371,7 @@ void hs_free(hs_handle* hd) {
   dev_free(hd, hd->ws64);
   dev_free(hd, hd->d_state);
   dev_free(hd, hd->lz);
+  dev_free(hd, hd->sb_m);
   dev_free(hd, hd->d_smr_first);
   sb_graphs_release(hd, 0);
   sb_graphs_release(hd, 1);

@@ -158,6 +158,8 @@ struct hs_handle {
   cudaGraphExec_t sbgraph[2][3] = {{nullptr, nullptr, nullptr}, {nullptr, nullptr, nullptr}};
   int sbgraph_key[2][3][2] = {};
   void* sbgraph_ws[2] = {nullptr, nullptr};
+  // M_ii and 1 / M_ii of the FP64 superblock solves (2 n doubles)
+  double* sb_m = nullptr;
 
   // Lanczos workspace
   double* lz = nullptr; size_t lz_vectors = 0;

@@ -80,13 +80,25 @@ hs_status solve_t(hs_handle* hd, const T* b, const MinresVecs& v, double tol, lo
   const int gA = use4 ? grid_of(hd, kern_A4<T>(d4->geo.km), nt_a4<T>(), smA, d4->geo.npairs)
                       : grid_of(hd, kern_A<T>(g.km), NT_A, smA, g.npairs);
   const int gI = grid_of(hd, kern_R<T, PC, sb::ROWS_INIT>(), NT_R, smR, g.npairs);
-  const int gB = grid_of(hd, kern_R<T, PC, sb::ROWS_B>(), NT_R, smR, g.npairs);
+  // FP64: M_ii and its reciprocal kept in memory (without room for them, or for
+  // the identity, which needs none, pass B as below)
+  constexpr bool flat = sizeof(T) == 8;
+  constexpr bool keeps_m = flat && PC != 0;
+  if (keeps_m && !hd->sb_m &&
+      dev_alloc(hd, (void**)&hd->sb_m, sizeof(double) * 2 * (size_t)hd->n) != HS_OK)
+    hd->err.clear();
+  const bool use_flat = flat && (!keeps_m || hd->sb_m);
+  const auto kflat = sb::k_flat_B<keeps_m>;
+  const int gB = use_flat ? grid_of(hd, kflat, sb::NT_FLAT, 0, (int)(hd->n / 2 / sb::NT_FLAT) + 1)
+                          : grid_of(hd, kern_R<T, PC, sb::ROWS_B>(), NT_R, smR, g.npairs);
   if (gA < 1 || gI < 1 || gB < 1) return HS_OK;
   *used = true;
   sb::MinresArgs ma;
   ma.v = v;
   ma.st = hd->d_state;
   ma.partial = hd->d_partial;
+  ma.m = keeps_m ? hd->sb_m : nullptr;
+  ma.mi = ma.m ? hd->sb_m + hd->n : nullptr;
   // initial pass: q_1 = M^-1 b, beta_1, state
   ma.counter = hd->d_counter + 0;
   kern_R<T, PC, sb::ROWS_INIT>()<<<gI, NT_R, smR, hd->stream>>>(g, b, ma, tol, kmax, hd->d_sigma);
@@ -96,7 +108,7 @@ hs_status solve_t(hs_handle* hd, const T* b, const MinresVecs& v, double tol, lo
   // and this workspace
   cudaGraphExec_t& exec = hd->sbgraph[ti][PC];
   int* key = hd->sbgraph_key[ti][PC];
-  const int keyA = gA | (use4 ? 1 << 30 : 0);
+  const int keyA = gA | (use4 ? 1 << 30 : 0) | (use_flat ? 1 << 29 : 0);
   if (exec && (key[0] != keyA || key[1] != gB || hd->sbgraph_ws[ti] != v.q0)) {
     cudaGraphExecDestroy(exec);
     exec = nullptr;
@@ -116,7 +128,10 @@ hs_status solve_t(hs_handle* hd, const T* b, const MinresVecs& v, double tol, lo
                                                               hd->d_sigma, 1, mA);
         else
           kern_A<T>(g.km)<<<gA, NT_A, smA, cs>>>(g, nullptr, nullptr, hd->d_sigma, 1, mA);
-        kern_R<T, PC, sb::ROWS_B>()<<<gB, NT_R, smR, cs>>>(g, nullptr, mB, 0.0, 0, hd->d_sigma);
+        if (use_flat)
+          kflat<<<gB, sb::NT_FLAT, 0, cs>>>(hd->n / 2, mB);
+        else
+          kern_R<T, PC, sb::ROWS_B>()<<<gB, NT_R, smR, cs>>>(g, nullptr, mB, 0.0, 0, hd->d_sigma);
       }
       e = cudaStreamEndCapture(cs, &graph);
     }

@@ -43,6 +43,8 @@ struct MinresArgs {
   MinresState* st;
   double* partial;
   unsigned* counter;
+  double* m;     // M_ii and 1 / M_ii (FP64 solves; null: recomputed per row)
+  double* mi;
 };
 
 constexpr int MODE_HV = 0;       // plain product
@@ -305,7 +307,15 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 1 : 2) k_sbrows(Geo g, co
             // a_ii = sigma (Sec. II assumes a_ii != sigma)
             const bool zero = !(mm > mtiny);
             zm += zero ? T(1) : T(0);
-            const T q = zero ? T(0) : va[j] / mm;
+            T q;
+            if (sizeof(T) == 8 && ma.m) {
+              const double im = zero ? 0.0 : 1.0 / (double)mm;
+              ma.m[i] = (double)mm;
+              ma.mi[i] = im;
+              q = (T)((double)va[j] * im);
+            } else {
+              q = zero ? T(0) : va[j] / mm;
+            }
             ((T*)v.q1)[i] = q;
             ((T*)v.q0)[i] = T(0);
             ((T*)v.d0)[i] = T(0);
@@ -347,6 +357,81 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 1 : 2) k_sbrows(Geo g, co
       }
       *ma.st = S;
     }
+  }
+}
+
+// Pass B of Algorithm 2 in FP64 with M_ii and 1 / M_ii read from memory (M =
+// false: the identity): element-wise over flat rows, two at a time (n is even).
+// k_sbrows forms M per row with a square root and divides by it: some 30 more
+// FP64 instructions a row on a pipe of 2 lanes per cycle and SM, where two more
+// vectors cost 16 bytes of 88. FP64 stays the bound (10 instructions a row, 53
+// us at n = 2.7 M against 35 us for the 11 vectors): L = 24: an
+// iteration 405 -> 266 us, all of it here.
+constexpr int NT_FLAT = 256;
+template <bool M>
+__global__ void __launch_bounds__(NT_FLAT) k_flat_B(long long n2, MinresArgs ma) {
+  __shared__ double s_red[32 * 4];
+  __shared__ double s_c[8];
+  __shared__ long long s_k;
+  __shared__ int s_done, s_pending;
+  if (threadIdx.x == 0) {
+    const MinresState* st = ma.st;
+    s_done = st->done; s_pending = st->pending; s_k = st->k;
+    const double bk = st->beta;
+    s_c[0] = 1.0 / bk; s_c[1] = st->alpha / bk; s_c[2] = bk / st->beta_prev;
+    s_c[4] = st->cq; s_c[5] = st->cd1; s_c[6] = st->cd2; s_c[7] = st->tau;
+  }
+  __syncthreads();
+  if (s_done == 2) return;
+  const bool doQ = s_done == 0;        // done == 1: only the last d/x update is left
+  const bool doC = s_pending != 0;
+  const MinresVecs& v = ma.v;
+  const bool odd = (s_k & 1) != 0;
+  const double2* qc = (const double2*)(odd ? v.q1 : v.q0);   // q_k
+  double2* qn = (double2*)(odd ? v.q0 : v.q1);               // q_{k-1} -> q_{k+1}
+  const double2* pv = (const double2*)v.p;
+  const double2* dA = (const double2*)(odd ? v.d1 : v.d0);   // d_{k-2}
+  double2* dB = (double2*)(odd ? v.d0 : v.d1);               // d_{k-3} -> d_{k-1}
+  double2* xv = (double2*)v.x;
+  const double2* mv = (const double2*)ma.m;
+  const double2* miv = (const double2*)ma.mi;
+  const double c1 = s_c[0], c2 = s_c[1], c3 = s_c[2];
+  const double cq = s_c[4], cd1 = s_c[5], cd2 = s_c[6], tau = s_c[7];
+  double acc = 0.0;
+  for (long long i = blockIdx.x * (long long)NT_FLAT + threadIdx.x; i < n2;
+       i += (long long)gridDim.x * NT_FLAT) {
+    // every load before any arithmetic
+    const double2 qp = qn[i];
+    double2 a, b, x, p, q, mm, im;
+    if (doC) { a = dA[i]; b = dB[i]; x = xv[i]; }
+    if (doQ) {
+      p = pv[i];
+      q = qc[i];
+      if (M) { mm = mv[i]; im = miv[i]; }
+    }
+    if (doC) {
+      const double2 d = {cq * qp.x + cd1 * a.x + cd2 * b.x, cq * qp.y + cd1 * a.y + cd2 * b.y};
+      dB[i] = d;
+      xv[i] = make_double2(x.x + tau * d.x, x.y + tau * d.y);
+    }
+    if (doQ) {
+      const double zx = M ? p.x * im.x : p.x, zy = M ? p.y * im.y : p.y;
+      const double2 r = {zx * c1 - c2 * q.x - c3 * qp.x, zy * c1 - c2 * q.y - c3 * qp.y};
+      qn[i] = r;
+      acc += (M ? mm.x * r.x : r.x) * r.x;
+      acc += (M ? mm.y * r.y : r.y) * r.y;
+    }
+  }
+  double vv[1] = {acc}, tot[1];
+  if (last_cta_sum<1>(vv, s_red, ma.partial, ma.counter, tot) && threadIdx.x == 0) {
+    MinresState S = *ma.st;
+    if (doQ) {
+      givens_update(S, tot[0]);       // sets the pending update of iteration k
+    } else {
+      S.pending = 0;                  // the last update is applied
+      S.done = 2;
+    }
+    *ma.st = S;
   }
 }
 
