@@ -547,7 +547,7 @@ hs_status solve_smem_job(hs_handle* hd, const void* b, const MinresVecs& v, hs_d
   HS_CUDA_TRY(hd, cudaMemsetAsync(hd->d_counter + 10, 0, sizeof(unsigned), hd->stream));
   // generation slots start from zero for every solve (a stale generation left
   // by a previous solve must never read as an arrival)
-  HS_CUDA_TRY(hd, cudaMemsetAsync(hd->d_partial, 0, 2 * sizeof(SlotN) * G, hd->stream));
+  HS_CUDA_TRY(hd, cudaMemsetAsync(hd->d_partial, 0, SMEM_SLOT_BYTES * G, hd->stream));
   unsigned long long limit = 1ull << 22;
   if (const char* e = getenv("HS_BARRIER_LIMIT")) limit = strtoull(e, nullptr, 10);
   SmemJob job{hd->geo(), b, v.x, hd->d_state, hd->sigma, tol, kmax};
@@ -693,10 +693,10 @@ static int sb_choice(const hs_handle* hd) {
 // The one-reduction form (minres_pipe.cu) is the first choice for FP64 solves
 // with the identity or row-norm preconditioner while a CTA holds at most 1024
 // rows: there the second grid reduction of the two-reduction form is a third
-// of the iteration (measured at L = 14..18 on 152 SMs: 18.5 -> 14.2, 20.7 ->
-// 14.9 and 22.6 -> 18.9 us per iteration, the same iteration counts, true
-// residuals within 2x of the tolerance at 1e-12). With more rows per CTA the
-// extra FP64 vector work cancels the gain (L = 20 on 152 SMs, L = 16 on 6).
+// of the iteration (L = 14..18 on 152 SMs: 18.5 -> 9.3, 20.7 -> 9.5 and
+// 22.6 -> 16.7 us per iteration, the same iteration counts, true residuals
+// within 2x of the tolerance at 1e-12). With more rows per CTA the extra FP64
+// vector work cancels the gain (L = 20 on 152 SMs, L = 16 on 6).
 // Not for Jacobi, whose ill-conditioned recurrence lets the carried p drift
 // (true residuals 10-100x the tolerance), nor by default for FP32, whose
 // drift costs the refinement sweeps more than the faster iterations win.

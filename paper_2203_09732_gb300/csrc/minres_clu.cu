@@ -74,7 +74,7 @@ hs_status launch_rpt(hs_handle* hd, const SmemJob& job, int pc, int cs) {
 // FP64 at n = 12870 stays with the grid forms (pipe_choice). HS_MINRES_CLUSTER
 // sets the number of CTAs (a power of two, at most 16; 0: off).
 int clu_choice(long long n, int sms) {
-  if (n > CLU_ROWS_MAX) return 0;
+  if (n > CLU_ROWS) return 0;
   int cs = n <= 128 ? 1 : n <= 512 ? 2 : n <= 1024 ? 8 : 16;
   if (const char* e = getenv("HS_MINRES_CLUSTER")) cs = atoi(e);
   while (cs > sms) cs >>= 1;

@@ -33,7 +33,7 @@ constexpr int CLU_CW = 3;                       // control warps (warps 0, 1 and
 constexpr int CLU_NT = 32 * (CLU_NW + CLU_CW);
 constexpr int CLU_SIZE_MAX = 16;                // CTAs per cluster
 constexpr int CLU_RPT_MAX = 8;                  // rows per thread
-constexpr int CLU_ROWS_MAX = CLU_SIZE_MAX * 32 * CLU_NW * CLU_RPT_MAX;
+static_assert(CLU_ROWS == CLU_SIZE_MAX * 32 * CLU_NW * CLU_RPT_MAX, "rows of the largest cluster");
 // polls of an mbarrier before a wait gives up with HS_TIMEOUT
 constexpr unsigned CLU_WAIT_LIMIT = 1u << 22;
 
@@ -119,12 +119,6 @@ __device__ __forceinline__ void clu_send2(uint32_t dst, float v, float w, uint32
   asm volatile(
       "st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(dst),
       "r"(__float_as_uint(v)), "r"(__float_as_uint(w)), "r"(bar) : "memory");
-}
-template <typename T>
-__device__ __forceinline__ T warp_sum_all(T v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
 }
 
 // Rows per CTA. With two or more rows a thread holds pairs of consecutive rows
@@ -225,6 +219,99 @@ __device__ __forceinline__ void clu_givens(MinresState& S, double sumsq, double 
   if (fabs(S.phi) < S.tol_abs || bn == 0.0 || S.k > S.kmax) S.done = 1;
 }
 
+constexpr int PIPE_NV = 5;           // S1..S5 (S6 is carried)
+
+// Smallest beta_{k+1}^2 / mag (mag: the sum of the expansion's terms in
+// magnitude) that the expansion is trusted with: its relative error is about
+// u mag / beta_{k+1}^2, at most 1e-8 (FP64) or 6e-5 (FP32) above the floor.
+// Below it (in practice: a Krylov space that has run out, as for n <= 8 or a
+// right-hand side inside an invariant subspace) the solve is handed back.
+template <typename T>
+constexpr double EXPANSION_FLOOR = sizeof(T) == 8 ? 1e-8 : 1e-3;
+
+// The scalars of step k of the one-reduction form, by one warp: from the sums
+// S1..S6, alpha_k, a = alpha_k / beta_k, c = beta_k / beta_{k-1} and the reciprocals
+// ib = 1 / beta_k, ib2 = ib^2, ibp = 1 / beta_{k-1}: beta_{k+1}, the Givens rotation;
+// ib and ibp move on a step. An FP64 instruction takes 64 cycles however many
+// lanes want it, so each term of beta_{k+1}^2 has a lane: 31 of them instead of
+// about 85 on one thread.
+template <typename T>
+__device__ __forceinline__ void pipe_scalars(MinresState& S, double S1, double S2, double S3,
+                                             double S4, double S5, double S6, double alpha, double a,
+                                             double c, double& ib, double ib2, double& ibp) {
+  constexpr unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31, tl = lane & 7;
+  // S2 / beta_k^2 | c^2 | c / beta_k
+  const double r = (tl == 0 ? S2 : c) * (tl == 0 ? ib2 : tl == 1 ? c : ib);
+  const double t1 = __shfl_sync(full, r, 0), cc = __shfl_sync(full, r, 1);
+  const double cb = __shfl_sync(full, r, 2);
+  // the terms, lanes 0..5 and, in magnitude, 8..13: S2 / beta^2, a^2 S4, c^2 S6,
+  // -2 a S1 / beta, -2 c S3 / beta, 2 a c S5
+  const double u = tl == 0 ? t1 : tl == 2 ? cc : tl == 4 ? cb : tl < 6 ? a : 0.0;
+  const double v = tl == 1 ? a : tl == 3 ? ib : tl == 5 ? c : 1.0;
+  const double w = tl == 1 ? S4 : tl == 2 ? S6 : tl == 3 ? S1 : tl == 4 ? S3 : tl == 5 ? S5 : 1.0;
+  const double f = tl < 3 ? 1.0 : tl < 5 ? -2.0 : 2.0;
+  double term = (u * v) * (w * f);
+  if (lane & 8) term = fabs(term);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) term += __shfl_xor_sync(full, term, o);
+  // b2 carries a rounding error of about u mag, with mag the sum of the terms'
+  // magnitudes and u the unit roundoff of the vectors
+  const double b2 = __shfl_sync(full, term, 0), mag = __shfl_sync(full, term, 8);
+  S.alpha = alpha;
+  S.pending = 0;
+  if (!isfinite(alpha) || !isfinite(b2)) {
+    S.status = HS_NONFINITE; S.done = 2;
+  } else if (!(b2 > EXPANSION_FLOOR<T> * mag)) {
+    S.status = HS_BREAKDOWN; S.pad = PIPE_EXPANSION; S.done = 2;
+  } else {
+    const double ibn = rsqrt(b2);
+    clu_givens(S, b2, b2 * ibn, ib);
+    ibp = ib;
+    ib = ibn;
+  }
+}
+
+// The block of row i, among blocks lo .. hi: the last one that starts at or
+// before it.
+__device__ __forceinline__ int clu_block(const Geo& g, uint32_t i, int lo, int hi) {
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (__ldg(&g.blocks[mid].R) <= i) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
+// Row i of H from the block tables (its block among lo .. hi): am = a_ii - sigma,
+// naf = its antiparallel bonds, put(r) for the row r at the other end of each.
+template <typename T, class F>
+__device__ __forceinline__ void clu_row(const Geo& g, uint32_t i, int lo, int hi, double sigma, T& am,
+                                        int& naf, F&& put) {
+  lo = clu_block(g, i, lo, hi);
+  const uint32_t* bw = reinterpret_cast<const uint32_t*>(g.blocks + lo);
+  Hdr h;
+  h.R = __ldg(bw);
+  h.Rwrap = __ldg(bw + 1);
+  h.bdelta = (int32_t)__ldg(bw + 2);
+  const uint32_t meta = __ldg(bw + 3);
+  h.w = meta & 0xFF;
+  h.nh = (meta >> 8) & 0xFF;
+  h.code = (meta >> 16) & 0xFF;
+  h.off = g.cls_off[h.w];
+  h.dhs = __hiloint2double((int)__ldg(bw + 5), (int)__ldg(bw + 4)) - sigma;
+  h.dhs_f = (float)h.dhs;
+  const LowEntry e = g.low[h.off + (int)(i - h.R)];
+  const uint32_t xc = cut_mask(e.packed, h);
+  for (int b = 0; b < le_cnt(e.packed); ++b)
+    put(h.R + ((e.nbw[b >> 2] >> (8 * (b & 3))) & 0xFFu));
+  for (int b = 0; b < h.nh; ++b) put((uint32_t)((int)i + (int)__ldg(bw + 6 + b)));
+  if (xc & 1u) put((uint32_t)((int)i + h.bdelta));
+  if (xc & 2u) put(h.Rwrap + e.wrap_r);
+  am = diag_t<T>(e, h, xc);
+  naf = naf_row(e.packed, h, xc);
+}
+
 // One solve by one cluster; every thread of every CTA calls it with the same
 // job. Where trace is set, CTA 0 writes alpha_k to trace[2 (k - 1)] and beta_{k+1}
 // to trace[2 (k - 1) + 1] (k = 1 .. kmax): the tridiagonal matrix of the Lanczos
@@ -295,39 +382,13 @@ __device__ bool clu_solve(const SmemJob& job, int pc, CluShared& sh, char* dyn, 
       int cnt = 0;
       if (owned(j)) {
         const uint32_t i = (uint32_t)(r0 + lrow(j));
-        // the row's block: the last one that starts at or before it
-        int lo = 0, hi = g.nblocks - 1;
-        while (lo < hi) {
-          const int mid = (lo + hi + 1) >> 1;
-          if (__ldg(&g.blocks[mid].R) <= i) lo = mid;
-          else hi = mid - 1;
-        }
-        const uint32_t* bw = reinterpret_cast<const uint32_t*>(g.blocks + lo);
-        Hdr h;
-        h.R = __ldg(bw);
-        h.Rwrap = __ldg(bw + 1);
-        h.bdelta = (int32_t)__ldg(bw + 2);
-        const uint32_t meta = __ldg(bw + 3);
-        h.w = meta & 0xFF;
-        h.nh = (meta >> 8) & 0xFF;
-        h.code = (meta >> 16) & 0xFF;
-        h.off = g.cls_off[h.w];
-        h.dhs = __hiloint2double((int)__ldg(bw + 5), (int)__ldg(bw + 4)) - sigma;
-        h.dhs_f = (float)h.dhs;
-        const LowEntry e = g.low[h.off + (int)(i - h.R)];
-        const uint32_t xc = cut_mask(e.packed, h);
         uint16_t* out = reinterpret_cast<uint16_t*>(nbr);
-        auto put = [&](uint32_t r) {
+        T am;
+        int naf;
+        clu_row<T>(g, i, 0, g.nblocks - 1, sigma, am, naf, [&](uint32_t r) {
           out[((cnt >> 1) * SLOTS + slot) * 2 + (cnt & 1)] = (uint16_t)r;
           ++cnt;
-        };
-        for (int b = 0; b < le_cnt(e.packed); ++b)
-          put(h.R + ((e.nbw[b >> 2] >> (8 * (b & 3))) & 0xFFu));
-        for (int b = 0; b < h.nh; ++b) put((uint32_t)((int)i + (int)__ldg(bw + 6 + b)));
-        if (xc & 1u) put((uint32_t)((int)i + h.bdelta));
-        if (xc & 2u) put(h.Rwrap + e.wrap_r);
-        const T am = diag_t<T>(e, h, xc);
-        const int naf = naf_row(e.packed, h, xc);
+        });
         const T mm = pc == 0 ? precond_t<0, T>(am, naf)
                    : pc == 1 ? precond_t<1, T>(am, naf) : precond_t<2, T>(am, naf);
         const T b = reinterpret_cast<const T*>(job.b)[i];

@@ -49,7 +49,8 @@ __device__ __forceinline__ void st_release_u32(unsigned* p, unsigned v) {
 // Rows of one block whose own segment (self and low-interior neighbours) is
 // read from shared memory xl; the other gathers come from global xg.
 // The rows are lane + 32 (j0 + j), j < JM: the block's 32-row chunks j0 on.
-template <typename T, int JM>
+// HG bonds' loads are in flight together.
+template <typename T, int JM, int HG = 4>
 __device__ __forceinline__ void block_hv_loc(const T* __restrict__ xg, const T* xl, const T* dg,
                                              const LowEntry* low, const Hdr& h, T (&xi)[JM],
                                              T (&hx)[JM], int j0 = 0) {
@@ -71,7 +72,6 @@ __device__ __forceinline__ void block_hv_loc(const T* __restrict__ xg, const T* 
       side[j] = c1 + c2;
     }
   }
-  constexpr int HG = 4;
   for (int m0 = 0; m0 < h.nh; m0 += HG) {
     T v[HG][JM];
 #pragma unroll
@@ -254,22 +254,110 @@ __device__ __forceinline__ void givens_fast(MinresState& S, double sumsq, double
 }
 
 
-// Reduction of NV <= SLOTN_VALS values: slot of one CTA (64 bytes).
-constexpr int SLOTN_VALS = 6;
-struct SlotN {
-  double v[SLOTN_VALS];
-  unsigned gen;
-  unsigned pad[3];
-};
+// Sum over a warp, in every lane.
+template <typename T>
+__device__ __forceinline__ T warp_sum_all(T v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
 
-// CTA-wide sums of NV per-thread values into sout[0..NV-1] (shared memory),
-// visible to every thread on return. Only the first nact warps hold values.
-// FP32 values are summed in FP32 within a warp and in FP64 across warps; FP64
-// values are staged in shared memory (stmp: NV * blockDim.x doubles) and
-// warp j adds value j, so the FP64 additions spread over NV warps.
+// A partial sum and the generation that marks it as published, moved in one
+// 16-byte access: a poll that sees the generation has the value.
+struct alignas(16) GridWord {
+  double v;
+  unsigned long long gen;
+};
+constexpr int GRID_WORDS = 3;    // words per CTA of one grid_total
+
+template <bool REL>
+__device__ __forceinline__ void word_store(GridWord* p, double v, unsigned long long gen) {
+  if constexpr (REL)
+    asm volatile("{\n.reg .b128 t;\nmov.b128 t, {%1, %2};\nst.release.gpu.global.b128 [%0], t;\n}" ::"l"(
+                     p), "l"(__double_as_longlong(v)), "l"(gen) : "memory");
+  else
+    asm volatile("{\n.reg .b128 t;\nmov.b128 t, {%1, %2};\nst.relaxed.gpu.global.b128 [%0], t;\n}" ::"l"(
+                     p), "l"(__double_as_longlong(v)), "l"(gen) : "memory");
+}
+template <bool ACQ>
+__device__ __forceinline__ double word_load(const GridWord* p, unsigned long long& gen) {
+  long long v;
+  if constexpr (ACQ)
+    asm volatile("{\n.reg .b128 t;\nld.acquire.gpu.global.b128 t, [%2];\nmov.b128 {%0, %1}, t;\n}"
+                 : "=l"(v), "=l"(gen) : "l"(p) : "memory");
+  else
+    asm volatile("{\n.reg .b128 t;\nld.relaxed.gpu.global.b128 t, [%2];\nmov.b128 {%0, %1}, t;\n}"
+                 : "=l"(v), "=l"(gen) : "l"(p) : "memory");
+  return __longlong_as_double(v);
+}
+
+// The grid's total of one value per CTA, by one warp of each CTA: the CTAs
+// publish their values in slots[0, G); CTA 0 adds them in a fixed order and
+// answers in slots[G + 2 c] (a 32-byte sector per CTA). False when the wait
+// gave up. ORD: what the CTAs stored to global memory before the call is
+// visible to all of them after it; without it the exchange carries the sum
+// only, and needs no fences (they double its time). Measured on 152 CTAs,
+// cycles: every CTA polling every CTA's word 7000-8600 (the words are a hot spot
+// of L2), this way 3500-4000, with the order 4200-5700; one way through L2 is
+// 600 (same die) to 980.
+template <bool ORD>
+__device__ __forceinline__ bool grid_total(GridWord* slots, int G, int cta, unsigned long long gen,
+                                          double mine, double& tot, unsigned long long limit,
+                                          int* err) {
+  const int lane = threadIdx.x & 31;
+  int ok = 1;
+  if (cta == 0) {
+    double v[8];
+    for (unsigned long long it = 0;;) {
+      bool all = true;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int c = lane + 32 * i;
+        v[i] = c == 0 ? mine : 0.0;
+        if (c > 0 && c < G) {
+          unsigned long long g;
+          v[i] = word_load<false>(slots + c, g);
+          all = all && g == gen;
+        }
+      }
+      if (__all_sync(0xffffffffu, all)) break;
+      if (++it > limit) { ok = 0; if (lane == 0) atomicExch(err, 1); break; }
+      if ((it & 255ull) == 0 && ld_relaxed_i32(err)) { ok = 0; break; }
+    }
+    ok = __all_sync(0xffffffffu, ok);
+    if (ok) {
+      double s = v[0];
+#pragma unroll
+      for (int i = 1; i < 8; ++i)
+        if (32 * i < G) s += v[i];
+      if (ORD) asm volatile("fence.acq_rel.gpu;" ::: "memory");
+      tot = warp_sum_all(s);
+      for (int c = lane; c < G; c += 32)
+        if (c > 0) word_store<false>(slots + G + 2 * c, tot, gen);
+    }
+  } else {
+    if (lane == 0) word_store<ORD>(slots + cta, mine, gen);
+    for (unsigned long long it = 0;;) {
+      unsigned long long g;
+      tot = word_load<ORD>(slots + G + 2 * cta, g);
+      if (__all_sync(0xffffffffu, g == gen)) break;
+      if (++it > limit) { ok = 0; if (lane == 0) atomicExch(err, 1); break; }
+      if ((it & 255ull) == 0 && ld_relaxed_i32(err)) { ok = 0; break; }
+    }
+    ok = __all_sync(0xffffffffu, ok);
+  }
+  return ok != 0;
+}
+
+// Sums over the CTA of NV per-thread values, value j in all lanes of warp j
+// (elsewhere 0). Only the first nact warps hold values. FP32 values are summed
+// in FP32 within a warp and in FP64 across warps; FP64 values are staged in
+// shared memory (stmp: NV * blockDim.x doubles) and warp j adds value j, so the
+// FP64 additions spread over NV warps.
 template <typename T, int NV>
-__device__ __forceinline__ void cta_sumN(const T (&a)[NV], int nact, double* stmp, double* sout) {
+__device__ __forceinline__ double cta_sumN(const T (&a)[NV], int nact, double* stmp) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  double t = 0.0;
   if constexpr (sizeof(T) == 4) {
 #pragma unroll
     for (int j = 0; j < NV; ++j) {
@@ -279,82 +367,26 @@ __device__ __forceinline__ void cta_sumN(const T (&a)[NV], int nact, double* stm
       if (lane == 0 && wid < nact) stmp[j * 32 + wid] = (double)v;
     }
     __syncthreads();
-    if (wid < NV) {
-      double t = lane < nact ? stmp[wid * 32 + lane] : 0.0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      if (lane == 0) sout[wid] = t;
-    }
+    if (wid < NV) t = lane < nact ? stmp[wid * 32 + lane] : 0.0;
   } else {
     const int nt = blockDim.x;
     if (wid < nact)
 #pragma unroll
       for (int j = 0; j < NV; ++j) stmp[j * nt + threadIdx.x] = a[j];
     __syncthreads();
-    if (wid < NV) {
-      double t = 0.0;
+    if (wid < NV)
       for (int i = lane; i < nact * 32; i += 32) t += stmp[wid * nt + i];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      if (lane == 0) sout[wid] = t;
-    }
   }
-  __syncthreads();
+  if (wid < NV)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return t;
 }
 
-// The slot reduction of slot_reduce_w0 for NV values (grids of at most 256
-// CTAs), called by warp 0 with the CTA's sums in c (shared memory): publish
-// with a release store of the generation, poll every slot with relaxed loads
-// (bounded by limit), one acquire fence, then a fixed-order sum so that every
-// CTA ends with identical totals in tot (all lanes).
-template <int NV>
-__device__ __forceinline__ bool slot_reduceN_w0(SlotN* slots, int G, int cta, unsigned gen,
-                                                const double* c, double (&tot)[NV],
-                                                unsigned long long limit, int* err) {
-  const int lane = threadIdx.x & 31;
-  SlotN* buf = slots + (size_t)(gen & 1u) * G;
-  if (lane == 0) {
-#pragma unroll
-    for (int j = 0; j < NV; ++j) buf[cta].v[j] = c[j];
-    st_release_u32(&buf[cta].gen, gen);
-  }
-  int ok = 1;
-  unsigned long long it = 0;
-  while (true) {
-    unsigned gv[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int cc = lane + 32 * q;
-      gv[q] = cc < G ? ld_relaxed_u32(&buf[cc].gen) : gen;
-    }
-    bool mine = true;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) mine = mine && (gv[q] == gen);
-    if (__all_sync(0xffffffffu, mine)) break;
-    if (++it > limit) { ok = 0; if (lane == 0) atomicExch(err, 1); break; }
-    if ((it & 255ull) == 0 && ld_relaxed_i32(err)) { ok = 0; break; }
-  }
-  asm volatile("fence.acq_rel.gpu;" ::: "memory");
-  double acc[NV];
-#pragma unroll
-  for (int j = 0; j < NV; ++j) acc[j] = 0.0;
-  if (ok) {
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int cc = lane + 32 * q;
-      if (cc < G)
-#pragma unroll
-        for (int j = 0; j < NV; ++j) acc[j] += __ldcg(&buf[cc].v[j]);
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < NV; ++j) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
-    tot[j] = acc[j];
-  }
-  return __all_sync(0xffffffffu, ok) != 0;
-}
+// Reduction slots of a shared-memory form, bytes per CTA: five exchanges of the
+// one-reduction form, two buffers of Slot of the other.
+constexpr size_t SMEM_SLOT_BYTES = 5 * GRID_WORDS * sizeof(GridWord);
+static_assert(SMEM_SLOT_BYTES >= 2 * sizeof(Slot), "slots of either form");
 
 // One solve of a job queue: the realisation's geometry, right-hand side and
 // solution (device, n elements of the solver's type), final state and
@@ -377,7 +409,7 @@ constexpr size_t SMEM_STATIC_BYTES = sizeof(MinresState) + sizeof(SmemJob) + 32 
 // jobs, both set before the launch); jobs == nullptr runs the kernel parameter
 // job0 alone, with one group. All jobs of a queue have the same L (one block
 // plan, cta_first, for the S CTAs of any group; nlow low-table entries).
-// slots: 2 S reduction slots per group; w[0..2]: the group's global vectors
+// slots: S * SMEM_SLOT_BYTES of reduction slots per group; w[0..2]: the group's global vectors
 // for the gathers, group g at w[i] + g ws_stride elements. Waits give up after
 // limit polls and set *err. A launch serves up to two queues (two chain
 // lengths): its first ctas0 CTAs take queue 0, the rest queue 1.
@@ -715,8 +747,8 @@ hs_status solve_clu(hs_handle* hd, const void* b, void* x, hs_dtype dt, int pc, 
 // j tstride. Asynchronous.
 hs_status launch_clu_many(const SmemJob* jobs, int count, int n, int L, int pc, int cs,
                           cudaStream_t s, double* trace, long long tstride);
-// FP64 solves of at most this many rows run in a cluster.
-constexpr long long CLU_F64_ROWS = 4096;
+// Solves of at most this many rows run in a cluster (in FP64, and in FP32).
+constexpr long long CLU_F64_ROWS = 4096, CLU_ROWS = 16384;
 
 // Contiguous block ranges per CTA with balanced row counts, cached per grid
 // size (minres.cu).

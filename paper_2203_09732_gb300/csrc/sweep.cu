@@ -87,7 +87,7 @@ struct Class {
   int* first = nullptr;
   int rows_cap = 0, hdr_cap = 0;
   int cap = 0;                       // job capacity
-  SlotN* slots = nullptr;
+  char* slots = nullptr;             // SMEM_SLOT_BYTES per CTA
   double* ws = nullptr;
   SmemJob* jobs = nullptr;
   MinresState* states = nullptr;
@@ -111,8 +111,7 @@ void free_class(Class& c) {
 
 hs_status alloc_class(Class& c, int num_sms) {
   c.cap = std::max((int)c.idx.size(), num_sms);
-  const size_t nslot = 2 * (size_t)num_sms;
-  if (cudaMalloc(&c.slots, nslot * sizeof(SlotN)) != cudaSuccess ||
+  if (cudaMalloc(&c.slots, SMEM_SLOT_BYTES * num_sms) != cudaSuccess ||
       cudaMalloc(&c.ws, 3 * (size_t)c.n * num_sms * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&c.jobs, c.cap * sizeof(SmemJob)) != cudaSuccess ||
       cudaMalloc(&c.states, c.cap * sizeof(MinresState)) != cudaSuccess ||
@@ -215,7 +214,7 @@ double time_groups(Class& c, const std::vector<LzRun>& runs, int pc, int S, bool
           cudaSuccess &&
       cudaMemcpyAsync(c.head, c.h_head, 2 * sizeof(int), cudaMemcpyHostToDevice, s) ==
           cudaSuccess &&
-      cudaMemsetAsync(c.slots, 0, 2 * (size_t)S * groups * sizeof(SlotN), s) == cudaSuccess &&
+      cudaMemsetAsync(c.slots, 0, SMEM_SLOT_BYTES * S * groups, s) == cudaSuccess &&
       cudaMemsetAsync(err, 0, sizeof(int), s) == cudaSuccess) {
     cudaEventRecord(e0, s);
     const hs_status ls = launch_pair(&c, nullptr, pc, one, c.hd0->k, device, s, err, 1ull << 22);
@@ -1145,7 +1144,7 @@ extern "C" hs_status hs_sweep(int B, const int* L_host, const double* h_host, in
       q[c] = make_queue(C, C.tune.S, err, limit);
       ng[c] = C.ngroups;
       hc[c] = C.hdr_cap;
-      if (cudaMemsetAsync(C.slots, 0, 2 * (size_t)num_sms * sizeof(SlotN), s) != cudaSuccess ||
+      if (cudaMemsetAsync(C.slots, 0, SMEM_SLOT_BYTES * num_sms, s) != cudaSuccess ||
           cudaMemsetAsync(dv[c].vgen, 0, sizeof(unsigned) * 2 * (size_t)num_sms, s) !=
               cudaSuccess) {
         cudaGetLastError();
