@@ -721,6 +721,14 @@ static int cluster_choice(const hs_handle* hd, bool f64, int pc) {
   return clu_choice(hd->n, std::max(1, std::min(hd->num_sms, bud > 0 ? bud : hd->num_sms)));
 }
 
+// The row form (minres_row.cu) takes what a cluster cannot hold, where a CTA's
+// rows fit its threads (L = 18 and 20 on the whole GPU). Not where another
+// form is asked for. HS_MINRES_ROW=0 / 1: off, or wherever it fits.
+static bool row_choice(const hs_handle* hd) {
+  if (const char* e = getenv("HS_MINRES_ROW")) return e[0] == '1';
+  return !getenv("HS_MINRES_PIPE") && hd->n > CLU_ROWS;
+}
+
 template <typename T, int PC>
 static hs_status try_sb(hs_handle* hd, const T* b, const MinresVecs& v, double tol,
                         long long kmax) {
@@ -744,6 +752,9 @@ static hs_status solve_pc(hs_handle* hd, const T* b, T* x, double tol, long long
                      ? cluster_choice(hd, sizeof(T) == 8, PC) : 0;
   if (cs > 0 && (st = solve_clu(hd, b, v.x, sizeof(T) == 8 ? HS_F64 : HS_F32, PC, tol, kmax,
                                 cs)) != HS_CUDA)
+    form = HS_FORM_SMEM;
+  if (st == HS_CUDA && !force_graph() && !force_global() && row_choice(hd) &&
+      (st = solve_row(hd, b, v, sizeof(T) == 8 ? HS_F64 : HS_F32, PC, tol, kmax)) != HS_CUDA)
     form = HS_FORM_SMEM;
   if (st == HS_CUDA && !force_graph() && !force_global() && pipe_choice(hd, sizeof(T) == 8, PC) &&
       (st = solve_smem_job(hd, b, v, sizeof(T) == 8 ? HS_F64 : HS_F32, PC, tol, kmax, true)) !=

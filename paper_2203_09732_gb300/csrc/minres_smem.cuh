@@ -747,6 +747,10 @@ hs_status solve_clu(hs_handle* hd, const void* b, void* x, hs_dtype dt, int pc, 
 // j tstride. Asynchronous.
 hs_status launch_clu_many(const SmemJob* jobs, int count, int n, int L, int pc, int cs,
                           cudaStream_t s, double* trace, long long tstride);
+// minres_row.cu: the row form (one solve on the handle's SMs, x in v.x, the
+// state in hd->h_state); HS_CUDA without a message when it does not apply.
+hs_status solve_row(hs_handle* hd, const void* b, const MinresVecs& v, hs_dtype dt, int pc,
+                    double tol, long long kmax);
 // Solves of at most this many rows run in a cluster (in FP64, and in FP32).
 constexpr long long CLU_F64_ROWS = 4096, CLU_ROWS = 16384;
 
