@@ -27,9 +27,10 @@
 
 #include "../../include/hs.h"
 
-// hv_sb.cu: whether the four-low-bit superblock form (sb4.cuh) serves products
-// and MINRES pass A of precision dt where its plan applies
-bool hs_want_sb4(hs_dtype dt);
+// hv_sb.cu: the superblock form that serves products and MINRES pass A of
+// precision dt where its plan applies: 6 or 4 low bits (sb6.cuh, sb4.cuh), or
+// ten (sb.cuh)
+int hs_want_sb(hs_dtype dt);
 
 namespace hs {
 
@@ -153,6 +154,8 @@ struct hs_handle {
   void* sb_plan[2] = {nullptr, nullptr};
   // four-low-bit superblock plans (sb4.cuh): [0] FP32, [1] FP64
   void* sb4_plan[2] = {nullptr, nullptr};
+  // six-low-bit superblock plan (sb6.cuh, FP64)
+  void* sb6_plan = nullptr;
   // superblock MINRES chunk graphs (minres_sb.cu), [precision][preconditioner],
   // with the grids (pass A, pass B) and the workspace they were captured for
   cudaGraphExec_t sbgraph[2][3] = {{nullptr, nullptr, nullptr}, {nullptr, nullptr, nullptr}};

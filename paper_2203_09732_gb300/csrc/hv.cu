@@ -157,13 +157,12 @@ static hs_status prep_smem(hs_handle* hd, K kern, size_t bytes) {
 
 hs_status launch_matvec(hs_handle* hd, const void* x, void* y, hs_dtype dt, int shifted) {
   {
-    // superblock forms from L = 24 on: in FP32 the ten-low-bit form (1.2-1.3x
-    // faster than the block form there), in FP64 the four-low-bit form (the
-    // FP64 pipe bounds every form; it does the fewest FP64 operations).
-    // HS_HV_SB=0 turns them off, =1 uses them wherever a plan was built
-    // (L >= 22).
+    // superblock forms: in FP32 from L = 24 on the ten-low-bit form (1.2-1.3x
+    // faster than the block form there), in FP64 from L = 22 on the six-low-bit
+    // form (L = 22 49 us against 55, L = 24 137 against 177). HS_HV_SB=0 turns
+    // them off, =1 uses them wherever a plan was built (L >= 22).
     const char* e = getenv("HS_HV_SB");
-    const bool on = e ? e[0] == '1' : hd->L >= 24;
+    const bool on = e ? e[0] == '1' : hd->L >= (dt == HS_F64 ? 22 : 24);
     if (on) {
       bool used = false;
       hs_status st = launch_matvec_sb(hd, x, y, dt, shifted, &used);
@@ -243,11 +242,11 @@ hs_status resid64(hs_handle* hd, const double* b, const double* x, double* r, hs
   if (x_zero) {
     st = resid64_t<RES_ZERO>(hd, b, x, r, pc, grid, sm);
   } else {
-    // where a superblock FP64 product applies (L >= 24) it is faster than the
+    // where a superblock FP64 product applies (L >= 22) it is faster than the
     // block form's: form (H - sigma) x in r, then r = b - r with the sums
     const char* e = getenv("HS_HV_SB");
     bool used = false;
-    if (e ? e[0] == '1' : hd->L >= 24)
+    if (e ? e[0] == '1' : hd->L >= 22)
       if ((st = launch_matvec_sb(hd, x, r, HS_F64, 1, &used)) != HS_OK) return st;
     st = used ? resid64_t<RES_GIVEN>(hd, b, x, r, pc, grid, sm)
               : resid64_t<RES_PRODUCT>(hd, b, x, r, pc, grid, sm);

@@ -11,6 +11,7 @@
 #include "common.cuh"
 #include "sb.cuh"
 #include "sb4_kern.cuh"
+#include "sb6_kern.cuh"
 #include "sb_kern.cuh"
 
 namespace hs {
@@ -195,6 +196,70 @@ static hs_status make_dev4(hs_handle* hd, int KS, DevPlan4** out) {
 
 }  // namespace sb4
 
+namespace sb6 {
+
+template <typename T>
+static hs_status make_dev6(hs_handle* hd, int KS, DevPlan6** out) {
+  *out = nullptr;
+  HostPlan6<T> P;
+  if (!build_plan6<T>(hd->L, hd->h, KS, &P)) return HS_OK;
+  const sb::HostPlan& B = P.base;
+  auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
+  struct Part { const void* src; size_t bytes; size_t at; };
+  std::vector<Part> parts = {{B.sup.data(), B.sup.size() * sizeof(sb::Sup), 0},
+                             {P.pairs.data(), P.pairs.size() * sizeof(int4), 0},
+                             {P.slotmap.data(), P.slotmap.size() * sizeof(uint16_t), 0},
+                             {P.tasks.data(), P.tasks.size() * sizeof(uint16_t), 0},
+                             {P.dmid.data(), P.dmid.size() * sizeof(T), 0},
+                             {P.dl.data(), P.dl.size() * sizeof(T), 0}};
+  size_t total = 0;
+  for (Part& q : parts) {
+    q.at = total;
+    total += al(q.bytes);
+  }
+  std::vector<char> host(total, 0);
+  for (const Part& q : parts) std::memcpy(host.data() + q.at, q.src, q.bytes);
+  DevPlan6* d = new DevPlan6();
+  if (dev_alloc(hd, &d->mem, total) != HS_OK) {
+    delete d;
+    return fail(hd, HS_OOM, "superblock table allocation failed");
+  }
+  // pageable source: the copy is staged before the call returns
+  if (cudaMemcpyAsync(d->mem, host.data(), total, cudaMemcpyHostToDevice, hd->stream) != cudaSuccess) {
+    cudaGetLastError();
+    dev_free(hd, d->mem);
+    delete d;
+    return fail(hd, HS_CUDA, "superblock table upload failed");
+  }
+  char* base = static_cast<char*>(d->mem);
+  Geo6& g = d->geo;
+  g.sup = reinterpret_cast<const sb::Sup*>(base + parts[0].at);
+  g.pairs = reinterpret_cast<const int4*>(base + parts[1].at);
+  g.slotmap = reinterpret_cast<const uint16_t*>(base + parts[2].at);
+  g.tasks = reinterpret_cast<const uint16_t*>(base + parts[3].at);
+  g.dmid = base + parts[4].at;
+  g.dl = base + parts[5].at;
+  g.npairs = (int)P.pairs.size();
+  g.km = B.km;
+  for (int i = 0; i <= sb::WQ_MAX; ++i) g.slot_off[i] = P.slot_off[i];
+  d->smem = smem_bytes6<T>(g.km);
+  auto kern = kernel6<T, sb::MODE_HV>();
+  int nb = 0;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d->smem) ==
+          cudaSuccess &&
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, NT6, d->smem) == cudaSuccess &&
+      nb > 0) {
+    d->grid = std::min(g.npairs, nb * hd->num_sms);
+    d->ok = 1;
+  } else {
+    cudaGetLastError();
+  }
+  *out = d;
+  return HS_OK;
+}
+
+}  // namespace sb6
+
 // Superblock windows of k + 4 bits (16 slots of 256 rows per superblock: x
 // slots and sums of a pair take 65 KB in FP32, two CTAs per SM) and at most
 // L - 10 bits, so that a chain has at least 512 superblock pairs to spread
@@ -221,6 +286,15 @@ hs_status sb_setup(hs_handle* hd) {
   hd->sb4_plan[0] = d4;
   if ((st = sb4::make_dev4<double>(hd, k64, &d4)) != HS_OK) return st;
   hd->sb4_plan[1] = d4;
+  // six-low-bit plan (sb6.cuh, FP64): 13-bit windows (the slots and sums of a
+  // pair take 97 KB; 12 and 11 bits leave more whole-superblock bonds to global
+  // memory, L = 28: 2084 -> 2811 -> 3682 us); HS_SB6_KS overrides it (tests of
+  // small chains)
+  int j64 = std::min(13, hd->L - 6);
+  if (const char* e = getenv("HS_SB6_KS")) j64 = atoi(e);
+  sb6::DevPlan6* d6 = nullptr;
+  if ((st = sb6::make_dev6<double>(hd, j64, &d6)) != HS_OK) return st;
+  hd->sb6_plan = d6;
   return HS_OK;
 }
 
@@ -239,19 +313,25 @@ void sb_release(hs_handle* hd) {
     }
     hd->sb4_plan[i] = nullptr;
   }
+  if (auto* d6 = static_cast<sb6::DevPlan6*>(hd->sb6_plan)) {
+    dev_free(hd, d6->mem);
+    delete d6;
+  }
+  hd->sb6_plan = nullptr;
 }
 
 }  // namespace hs
 
-// The four-low-bit form is the FP64 default (measured at L = 24..28 it is the
-// fastest FP64 product: fewer FP64 additions of zeros than the ten-bit form,
-// and no gathers from global memory for most bonds, unlike the block form);
-// in FP32 the ten-bit form is faster. HS_SB4=1 / 0 selects it, or not, for
-// both precisions (tests compare forms).
-bool hs_want_sb4(hs_dtype dt) {
+// The low bits of the superblock form: six in FP64, whose additions bound every
+// form (the six-bit one adds the fewest: no zeros for parallel mid bonds, and the
+// fewest instructions around them; L = 24: 137 us, four bits 172, block 177; L = 28:
+// 2.08 ms, 2.50, 2.64), ten in FP32, where the gathers of the whole-superblock
+// bonds bound all of them (L = 28: 334 us, six bits 344, four 392). HS_SB4=1 / 0
+// selects four or ten bits for both (tests compare forms).
+int hs_want_sb(hs_dtype dt) {
   const char* e = getenv("HS_SB4");
-  if (e) return e[0] == '1';
-  return dt == HS_F64;
+  if (e) return e[0] == '1' ? 4 : 10;
+  return dt == HS_F64 ? 6 : 10;
 }
 
 namespace hs {
@@ -259,10 +339,24 @@ namespace hs {
 hs_status launch_matvec_sb(hs_handle* hd, const void* x, void* y, hs_dtype dt, int shifted,
                            bool* used) {
   *used = false;
+  const int want = hs_want_sb(dt);
+  {
+    auto* d6 = static_cast<sb6::DevPlan6*>(hd->sb6_plan);
+    if (want == 6 && d6 && d6->ok && ((uintptr_t)x % 8) == 0 && ((uintptr_t)y % 8) == 0) {
+      const sb::MinresArgs none{};
+      sb6::kernel6<double, sb::MODE_HV>()<<<d6->grid, sb6::NT6, d6->smem, hd->stream>>>(
+          d6->geo, static_cast<const double*>(x), static_cast<double*>(y), hd->d_sigma, shifted,
+          none);
+      count_launches(1);
+      HS_CUDA_TRY(hd, cudaGetLastError());
+      *used = true;
+      return HS_OK;
+    }
+  }
   {
     auto* d4 = static_cast<sb4::DevPlan4*>(hd->sb4_plan[dt == HS_F32 ? 0 : 1]);
     const size_t es = dt == HS_F32 ? sizeof(float) : sizeof(double);
-    if (hs_want_sb4(dt) && d4 && d4->ok && ((uintptr_t)x % es) == 0 && ((uintptr_t)y % es) == 0) {
+    if (want == 4 && d4 && d4->ok && ((uintptr_t)x % es) == 0 && ((uintptr_t)y % es) == 0) {
       const sb::MinresArgs none{};
       if (dt == HS_F32)
         sb4::kernel4_for<float, sb::MODE_HV>(d4->geo.km)<<<d4->grid, sb4::NT4_F, d4->smem,

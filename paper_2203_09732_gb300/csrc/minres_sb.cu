@@ -14,6 +14,7 @@
 #include "common.cuh"
 #include "minres_scalar.cuh"
 #include "sb4_kern.cuh"
+#include "sb6_kern.cuh"
 #include "sb_kern.cuh"
 
 namespace hs {
@@ -74,10 +75,15 @@ hs_status solve_t(hs_handle* hd, const T* b, const MinresVecs& v, double tol, lo
   if (!d || !d->ok) return HS_OK;
   const sb::Geo& g = d->geo;
   auto* d4 = static_cast<sb4::DevPlan4*>(hd->sb4_plan[ti]);
-  const bool use4 = hs_want_sb4(sizeof(T) == 8 ? HS_F64 : HS_F32) && d4 && d4->ok;
-  const size_t smA = use4 ? d4->smem : d->smem;
+  auto* d6 = static_cast<sb6::DevPlan6*>(hd->sb6_plan);
+  const int want = hs_want_sb(sizeof(T) == 8 ? HS_F64 : HS_F32);
+  const bool use4 = want == 4 && d4 && d4->ok;
+  const bool use6 = sizeof(T) == 8 && want == 6 && d6 && d6->ok;
+  const auto kA6 = sb6::kernel6<double, sb::MODE_MINRES>();
+  const size_t smA = use6 ? d6->smem : use4 ? d4->smem : d->smem;
   const size_t smR = sb::rows_smem_bytes<T>(1 << g.k);
-  const int gA = use4 ? grid_of(hd, kern_A4<T>(d4->geo.km), nt_a4<T>(), smA, d4->geo.npairs)
+  const int gA = use6 ? grid_of(hd, kA6, sb6::NT6, smA, d6->geo.npairs)
+               : use4 ? grid_of(hd, kern_A4<T>(d4->geo.km), nt_a4<T>(), smA, d4->geo.npairs)
                       : grid_of(hd, kern_A<T>(g.km), NT_A, smA, g.npairs);
   const int gI = grid_of(hd, kern_R<T, PC, sb::ROWS_INIT>(), NT_R, smR, g.npairs);
   // FP64: M_ii and its reciprocal kept in memory (without room for them, or for
@@ -108,7 +114,7 @@ hs_status solve_t(hs_handle* hd, const T* b, const MinresVecs& v, double tol, lo
   // and this workspace
   cudaGraphExec_t& exec = hd->sbgraph[ti][PC];
   int* key = hd->sbgraph_key[ti][PC];
-  const int keyA = gA | (use4 ? 1 << 30 : 0) | (use_flat ? 1 << 29 : 0);
+  const int keyA = gA | (use4 ? 1 << 30 : 0) | (use6 ? 1 << 28 : 0) | (use_flat ? 1 << 29 : 0);
   if (exec && (key[0] != keyA || key[1] != gB || hd->sbgraph_ws[ti] != v.q0)) {
     cudaGraphExecDestroy(exec);
     exec = nullptr;
@@ -123,7 +129,9 @@ hs_status solve_t(hs_handle* hd, const T* b, const MinresVecs& v, double tol, lo
       mA.counter = hd->d_counter + 1;
       mB.counter = hd->d_counter + 2;
       for (int it = 0; it < SB_CHUNK; ++it) {
-        if (use4)
+        if (use6)
+          kA6<<<gA, sb6::NT6, smA, cs>>>(d6->geo, nullptr, nullptr, hd->d_sigma, 1, mA);
+        else if (use4)
           kern_A4<T>(d4->geo.km)<<<gA, nt_a4<T>(), smA, cs>>>(d4->geo, nullptr, nullptr,
                                                               hd->d_sigma, 1, mA);
         else
