@@ -692,13 +692,14 @@ static int sb_choice(const hs_handle* hd, bool f64) {
   return hd->L >= (f64 ? 22 : 24) ? 1 : 0;
 }
 
-// The one-reduction form (minres_pipe.cu) is the first choice for FP64 solves
-// with the identity or row-norm preconditioner while a CTA holds at most 1024
-// rows: there the second grid reduction of the two-reduction form is a third
-// of the iteration (L = 14..18 on 152 SMs: 18.5 -> 9.3, 20.7 -> 9.5 and
-// 22.6 -> 16.7 us per iteration, the same iteration counts, true residuals
-// within 2x of the tolerance at 1e-12). With more rows per CTA the extra FP64
-// vector work cancels the gain (L = 20 on 152 SMs, L = 16 on 6).
+// The one-reduction recurrence is the first choice for FP64 solves with the
+// identity or row-norm preconditioner while a CTA holds at most 1024 rows, in
+// the row layout (minres_row1.cu) where that fits, else minres_pipe.cu: there the
+// second grid reduction is a third of the iteration (one against two reductions
+// in the row layout, us per iteration on 152 SMs: L = 14 6.0 against 9.6, L = 16
+// 6.3 against 9.6, L = 18 8.9 against 12.4; the same iteration counts, true
+// residuals within 2x of the tolerance at 1e-12). With more rows per CTA the
+// extra FP64 vector work cancels the gain (L = 20 on 152 SMs, L = 16 on 6).
 // Not for Jacobi, whose ill-conditioned recurrence lets the carried p drift
 // (true residuals 10-100x the tolerance), nor by default for FP32, whose
 // drift costs the refinement sweeps more than the faster iterations win.
@@ -706,6 +707,7 @@ static int sb_choice(const hs_handle* hd, bool f64) {
 static bool pipe_choice(const hs_handle* hd, bool f64, int pc) {
   const char* e = getenv("HS_MINRES_PIPE");
   if (e) return e[0] == '1';
+  if ((e = getenv("HS_MINRES_ROW")) && e[0] == '1') return false;
   if (!f64 || pc == 1) return false;
   const int bud = hd->sm_budget.load(std::memory_order_relaxed);
   const int G = std::max(1, std::min(hd->num_sms, bud > 0 ? bud : hd->num_sms));
@@ -724,7 +726,8 @@ static int cluster_choice(const hs_handle* hd, bool f64, int pc) {
 }
 
 // The row form (minres_row.cu) takes what a cluster cannot hold, where a CTA's
-// rows fit its threads (L = 18 and 20 on the whole GPU). Not where another
+// rows fit its threads (L = 18 and 20 on the whole GPU) and the one-reduction
+// recurrence is not taken. Not where another
 // form is asked for. HS_MINRES_ROW=0 / 1: off, or wherever it fits.
 static bool row_choice(const hs_handle* hd) {
   if (const char* e = getenv("HS_MINRES_ROW")) return e[0] == '1';
@@ -755,13 +758,16 @@ static hs_status solve_pc(hs_handle* hd, const T* b, T* x, double tol, long long
   if (cs > 0 && (st = solve_clu(hd, b, v.x, sizeof(T) == 8 ? HS_F64 : HS_F32, PC, tol, kmax,
                                 cs)) != HS_CUDA)
     form = HS_FORM_SMEM;
+  if (st == HS_CUDA && !force_graph() && !force_global() && pipe_choice(hd, sizeof(T) == 8, PC)) {
+    const hs_dtype dt = sizeof(T) == 8 ? HS_F64 : HS_F32;
+    bool broke = false;
+    st = solve_row1(hd, b, v, dt, PC, tol, kmax, &broke);
+    if (st == HS_CUDA && !broke) st = solve_smem_job(hd, b, v, dt, PC, tol, kmax, true);
+    if (st != HS_CUDA) form = HS_FORM_SMEM1;
+  }
   if (st == HS_CUDA && !force_graph() && !force_global() && row_choice(hd) &&
       (st = solve_row(hd, b, v, sizeof(T) == 8 ? HS_F64 : HS_F32, PC, tol, kmax)) != HS_CUDA)
     form = HS_FORM_SMEM;
-  if (st == HS_CUDA && !force_graph() && !force_global() && pipe_choice(hd, sizeof(T) == 8, PC) &&
-      (st = solve_smem_job(hd, b, v, sizeof(T) == 8 ? HS_F64 : HS_F32, PC, tol, kmax, true)) !=
-          HS_CUDA)
-    form = HS_FORM_SMEM1;
   if (st == HS_CUDA && !force_graph() && !force_global() &&
       (st = solve_smem<T, PC>(hd, b, v, tol, kmax)) != HS_CUDA)
     form = HS_FORM_SMEM;

@@ -751,6 +751,10 @@ hs_status launch_clu_many(const SmemJob* jobs, int count, int n, int L, int pc, 
 // state in hd->h_state); HS_CUDA without a message when it does not apply.
 hs_status solve_row(hs_handle* hd, const void* b, const MinresVecs& v, hs_dtype dt, int pc,
                     double tol, long long kmax);
+// minres_row1.cu: the one-reduction recurrence on the row layout, as solve_row;
+// HS_CUDA with *broke set where the expansion of beta_{k+1}^2 failed.
+hs_status solve_row1(hs_handle* hd, const void* b, const MinresVecs& v, hs_dtype dt, int pc,
+                     double tol, long long kmax, bool* broke);
 // Solves of at most this many rows run in a cluster (in FP64, and in FP32).
 constexpr long long CLU_F64_ROWS = 4096, CLU_ROWS = 16384;
 
