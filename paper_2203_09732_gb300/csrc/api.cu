@@ -106,6 +106,26 @@ uint32_t binom(int n, int r) {
   return (uint32_t)v;
 }
 
+// The low table followed by its sorted lists (LowSorted).
+static std::vector<LowEntry> with_sorted(const hs_handle* hd) {
+  const size_t nlow = hd->low.size();
+  std::vector<LowSorted> so(2 * ((nlow + 1) / 2));
+  const Geo g = hd->geo();
+  for (int w = 0; w <= g.k; ++w) {
+    int at = g.cls_off[w];
+    for (int cnt = NB_MAX; cnt >= 0; --cnt)
+      for (int r = 0; r < g.cls_C[w]; ++r) {
+        const LowEntry& e = hd->low[g.cls_off[w] + r];
+        if (le_cnt(e.packed) == cnt)
+          so[at++] = LowSorted{{e.nbw[0], e.nbw[1], e.nbw[2]}, (uint32_t)r | (uint32_t)cnt << 8};
+      }
+  }
+  std::vector<LowEntry> t(hd->low);
+  t.resize(nlow + so.size() / 2);
+  memcpy(t.data() + nlow, so.data(), so.size() * sizeof(LowSorted));
+  return t;
+}
+
 int row_grid(const hs_handle* hd) {
   const int need = ((int)hd->blocks.size() + HV_WARPS - 1) / HV_WARPS;
   return std::max(1, std::min(need, hd->grid_hv));
@@ -325,7 +345,7 @@ hs_status hs_create(int L, const double* h_host, double sigma, void* cuda_stream
   }
   hd->grid_hv = std::min(RED_MAX_CTAS, hd->num_sms * 4);
   if ((st = build_tables(hd)) != HS_OK) return bail(st);
-  if ((st = upload(hd, &hd->d_low, hd->low)) != HS_OK) return bail(st);
+  if ((st = upload(hd, &hd->d_low, with_sorted(hd))) != HS_OK) return bail(st);
   if ((st = upload(hd, &hd->d_blocks, hd->blocks)) != HS_OK) return bail(st);
   {
     const int W = LMAX / 2 + 2;

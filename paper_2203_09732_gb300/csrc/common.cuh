@@ -53,6 +53,14 @@ struct LowEntry {
   double dlow;       // Ising terms of low interior bonds + fields on low sites
 };
 static_assert(sizeof(LowEntry) == 32, "LowEntry is 32 bytes");
+// The low table is followed by one of these per entry: the entries of each class
+// in order of falling neighbour count, so that a warp's threads add about as
+// many neighbours.
+struct LowSorted {
+  uint32_t nbw[3];   // as in the entry of rank row in the class
+  uint32_t meta;     // row | nb_cnt << 8
+};
+static_assert(sizeof(LowSorted) == 16, "LowSorted is 16 bytes");
 // code = bit (k-1) of p | bit 0 of p << 1; tlow = sum of (j + 1) over set bits j < k.
 
 __host__ __device__ inline uint32_t le_pat(uint32_t pk) { return pk & 0xFFFFu; }

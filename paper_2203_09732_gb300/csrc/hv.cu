@@ -1,6 +1,7 @@
 // Matrix-free H x (Eq. (1)), the basis ranking (Sec. I: Sz = 0 sector in
 // ascending integer order), the diagonal / preconditioner export (Sec. II) and
 // the FP64 refinement residual r = b - (H - sigma) x.
+#include <algorithm>
 #include <cstdlib>
 
 #include "rows.cuh"
@@ -8,7 +9,8 @@
 namespace hs {
 
 // ---------------------------------------------------------------------------
-// y = (H - sigma * shifted) x. Warps walk the blocks in rank order.
+// y = (H - sigma * shifted) x. Warps walk the blocks in rank order. FP32 chains
+// without a superblock plan from L = 24 on.
 template <typename T>
 __global__ void __launch_bounds__(HV_THREADS) k_matvec(Geo g, const T* __restrict__ x,
                                                        T* __restrict__ y, const double* d_sigma,
@@ -25,6 +27,105 @@ __global__ void __launch_bounds__(HV_THREADS) k_matvec(Geo g, const T* __restric
     for (int j = 0; j < JMAX; ++j)
       if (j < h.J && lane + 32 * j < h.C) __stcs(yb + 32 * j, hx[j]);
   });
+}
+
+// v / 2. FP64: by the exponent where that is exact in every lane of the warp (a few
+// integer instructions instead of one on the FP64 pipe).
+__device__ __forceinline__ float half_of(float v) { return 0.5f * v; }
+__device__ __forceinline__ double half_of(double v) {
+  const int hi = __double2hiint(v), lo = __double2loint(v);
+  const uint32_t e = ((uint32_t)hi >> 20) & 0x7FFu;
+  const bool zero = ((uint32_t)(hi << 1) | (uint32_t)lo) == 0u;
+  if (!__all_sync(0xffffffffu, zero || e - 2u < 2045u)) return 0.5 * v;
+  return __hiloint2double(zero ? hi : hi - 0x100000, lo);
+}
+
+// y = (H - sigma * shifted) x, one thread per row and one CTA per block (as many
+// threads as the longest block has rows). Every load of a row but the low
+// neighbours (from the block's x segment in shared memory) goes out at once, so
+// a short chain costs a launch and three trips to L2; in FP64 the FP64 pipe
+// bounds the long ones (about 16 instructions a row at L = 24, 19 cycles per warp
+// and SM: 90 us), so nothing adds zeros, the low neighbours are summed by the
+// threads in the order of LowSorted (5 adds in a warp instead of 8) and the halving
+// is done on the exponent (without that and the votes on c1, c2: 119 and 469 us at
+// L = 24 and 26). k_matvec, with up to eight rows per lane, added zeros for rows and bonds that were not
+// there and copied the low table to each CTA. us, that form -> this (L = 24, 26
+// FP64: sb6 -> this; L = 24 before both 176):
+//   FP64  L = 12 8.2 -> 4.1  16 10.8 -> 5.2  20 31.1 -> 14.4  22 55 -> 35  24 137 -> 116  26 528 -> 445
+//   FP32  L = 12 6.2 -> 4.1  16 6.2 -> 4.1  20 8.2 -> 6.2  22 14.4 -> 12.3
+// 40 warps per SM in FP64 (48 registers): with 32 and 48 119 and 121 us at L = 24.
+template <typename T>
+__global__ void __launch_bounds__(32 * JMAX, sizeof(T) == 8 ? 5 : 6) k_rows(Geo g, const T* __restrict__ x,
+                                                    T* __restrict__ y, const double* d_sigma,
+                                                    int shifted) {
+  __shared__ T xs[32 * JMAX], ls[32 * JMAX], ds[4];
+  constexpr int HB = 10;                        // high bonds gathered at once
+  const uint4* hw = reinterpret_cast<const uint4*>(g.blocks + blockIdx.x);
+  const uint4 h0 = __ldg(hw), h1 = __ldg(hw + 1), h2 = __ldg(hw + 2), h3 = __ldg(hw + 3);
+  const int w = h0.w & 0xFF, nh = (h0.w >> 8) & 0xFF, code = (h0.w >> 16) & 3;
+  const int r = threadIdx.x, C = g.cls_C[w];
+  const bool on = r < C;
+  if (r < 4) {
+    // what a_ii - sigma has besides the entry's dlow, by cut bonds that flip
+    const double dhs = __hiloint2double((int)h1.y, (int)h1.x) - (shifted ? __ldg(d_sigma) : 0.0);
+    ds[r] = (T)dhs + (T(0.5) - T(0.5) * T(__popc(r)));
+  }
+  T xi = T(0), c1 = T(0), c2 = T(0), dlow = T(0);
+  uint4 so = make_uint4(0, 0, 0, 0);
+  uint32_t xc = 0;
+  const T* xr = x + h0.x + r;
+  T v[HB];
+  if (on) {
+    const LowEntry* le = g.low + g.cls_off[w] + r;
+    const uint2 e = __ldg(reinterpret_cast<const uint2*>(le));
+    so = __ldg(reinterpret_cast<const uint4*>(g.low + g.nlow) + g.cls_off[w] + r);
+    if constexpr (sizeof(T) == 8) dlow = __ldg(&le->dlow);
+    else dlow = __ldg(&le->dlow_f);
+    xi = __ldg(xr);
+    const uint32_t hd[HB] = {h1.z, h1.w, h2.x, h2.y, h2.z, h2.w, h3.x, h3.y, h3.z, h3.w};
+#pragma unroll
+    for (int m = 0; m < HB; ++m)
+      if (m < nh) v[m] = __ldg(xr + (int32_t)hd[m]);
+    xc = le_code(e.x) ^ code;
+    if (xc & 1u) c1 = __ldg(xr + (int32_t)h0.z);
+    if (xc & 2u) c2 = __ldg(x + (h0.y + (e.y & 0xFFFFu)));
+  }
+  xs[r] = xi;
+  __syncthreads();
+  // the low neighbours of the row that so names
+  const int cnt = so.w >> 8;
+  const int most = __reduce_max_sync(0xffffffffu, cnt);
+  T acc = T(0);
+#pragma unroll
+  for (int m = 0; m < NB_MAX; ++m) {
+    if (m >= most) break;
+    const uint32_t wd = m < 4 ? so.x : m < 8 ? so.y : so.z;
+    const uint32_t q = (wd >> (8 * (m & 3))) & 0xFFu;
+    if (m == 0) acc = cnt > 0 ? xs[q] : T(0);
+    else if (m < cnt) acc += xs[q];
+  }
+  if (on) ls[so.w & 0xFFu] = acc;
+  __syncthreads();
+  if ((r & ~31) >= C) return;
+  acc = on ? ls[r] : T(0);
+  for (int m0 = HB; m0 < nh; m0 += 4) {
+    const uint4 hh = __ldg(hw + 4 + ((m0 - HB) >> 2));
+    const uint32_t hd[4] = {hh.x, hh.y, hh.z, hh.w};
+    T u[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+      u[m] = on && m0 + m < nh ? __ldg(xr + (int32_t)hd[m]) : T(0);
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+      if (m0 + m < nh) acc += u[m];
+  }
+#pragma unroll
+  for (int m = 0; m < HB; ++m)
+    if (m < nh) acc += v[m];
+  if (__any_sync(0xffffffffu, xc & 1u)) acc += c1;
+  if (__any_sync(0xffffffffu, xc & 2u)) acc += c2;
+  const T half = half_of(acc);
+  if (on) __stcs(y + h0.x + r, (dlow + ds[xc]) * xi + half);
 }
 
 // ---------------------------------------------------------------------------
@@ -156,32 +257,33 @@ static hs_status prep_smem(hs_handle* hd, K kern, size_t bytes) {
 }
 
 hs_status launch_matvec(hs_handle* hd, const void* x, void* y, hs_dtype dt, int shifted) {
-  {
-    // superblock forms: in FP32 from L = 24 on the ten-low-bit form (1.2-1.3x
-    // faster than the block form there), in FP64 from L = 22 on the six-low-bit
-    // form (L = 22 49 us against 55, L = 24 137 against 177). HS_HV_SB=0 turns
-    // them off, =1 uses them wherever a plan was built (L >= 22).
-    const char* e = getenv("HS_HV_SB");
-    const bool on = e ? e[0] == '1' : hd->L >= (dt == HS_F64 ? 22 : 24);
-    if (on) {
-      bool used = false;
-      hs_status st = launch_matvec_sb(hd, x, y, dt, shifted, &used);
-      if (st != HS_OK || used) return st;
-    }
+  // FP64: one thread per row at every L (the six-low-bit superblock form takes
+  // 49, 137, 528 and 2084 us at L = 22 .. 28, this 35, 116, 445 and 1775). FP32:
+  // the ten-low-bit superblock form from L = 24 on (27, 82 and 333 us at L = 24,
+  // 26, 28; one thread per row 31, 123 and 600: its far gathers miss L2), and
+  // where it has no plan there the block form (36, 115, 498). HS_HV_SB=0 turns
+  // the superblock forms off, =1 uses them wherever a plan was built.
+  const char* e = getenv("HS_HV_SB");
+  if (e ? e[0] == '1' : hd->L >= 24 && dt == HS_F32) {
+    bool used = false;
+    hs_status st = launch_matvec_sb(hd, x, y, dt, shifted, &used);
+    if (st != HS_OK || used) return st;
   }
   const Geo g = hd->geo();
-  const int grid = row_grid(hd);
-  if (dt == HS_F32) {
+  const int nt = (*std::max_element(g.cls_C, g.cls_C + g.k + 1) + 31) / 32 * 32;
+  if (dt == HS_F64) {
+    k_rows<double><<<g.nblocks, nt, 0, hd->stream>>>(
+        g, static_cast<const double*>(x), static_cast<double*>(y), hd->d_sigma, shifted);
+  } else if (hd->L < 24) {
+    k_rows<float><<<g.nblocks, nt, 0, hd->stream>>>(
+        g, static_cast<const float*>(x), static_cast<float*>(y), hd->d_sigma, shifted);
+  } else {
     const size_t sm = smem_of<float>(hd);
     if (prep_smem(hd, k_matvec<float>, sm) != HS_OK) return HS_CUDA;
-    k_matvec<float><<<grid, HV_THREADS, sm, hd->stream>>>(
-        g, static_cast<const float*>(x), static_cast<float*>(y), hd->d_sigma, shifted); count_launches(1);
-  } else {
-    const size_t sm = smem_of<double>(hd);
-    if (prep_smem(hd, k_matvec<double>, sm) != HS_OK) return HS_CUDA;
-    k_matvec<double><<<grid, HV_THREADS, sm, hd->stream>>>(
-        g, static_cast<const double*>(x), static_cast<double*>(y), hd->d_sigma, shifted); count_launches(1);
+    k_matvec<float><<<row_grid(hd), HV_THREADS, sm, hd->stream>>>(
+        g, static_cast<const float*>(x), static_cast<float*>(y), hd->d_sigma, shifted);
   }
+  count_launches(1);
   HS_CUDA_TRY(hd, cudaGetLastError());
   return HS_OK;
 }
@@ -242,12 +344,16 @@ hs_status resid64(hs_handle* hd, const double* b, const double* x, double* r, hs
   if (x_zero) {
     st = resid64_t<RES_ZERO>(hd, b, x, r, pc, grid, sm);
   } else {
-    // where a superblock FP64 product applies (L >= 22) it is faster than the
-    // block form's: form (H - sigma) x in r, then r = b - r with the sums
+    // from L = 22 on the product kernel and a pass over its result are faster
+    // than both in the block form: form (H - sigma) x in r, then r = b - r with
+    // the sums
     const char* e = getenv("HS_HV_SB");
-    bool used = false;
-    if (e ? e[0] == '1' : hd->L >= 22)
-      if ((st = launch_matvec_sb(hd, x, r, HS_F64, 1, &used)) != HS_OK) return st;
+    bool used = !e && hd->L >= 22;
+    if (used)
+      st = launch_matvec(hd, x, r, HS_F64, 1);
+    else if (e && e[0] == '1')
+      st = launch_matvec_sb(hd, x, r, HS_F64, 1, &used);
+    if (st != HS_OK) return st;
     st = used ? resid64_t<RES_GIVEN>(hd, b, x, r, pc, grid, sm)
               : resid64_t<RES_PRODUCT>(hd, b, x, r, pc, grid, sm);
   }
