@@ -228,7 +228,7 @@ def peaks():
 
 def kernel_source_hash():
     h = hashlib.sha256()
-    for f in ("common.cuh", "sb.cuh", "sb_kern.cuh", "sb4.cuh", "sb4_kern.cuh", "hv_sb.cu"):
+    for f in ("common.cuh", "rows.cuh", "hv_cls.cuh"):
         h.update(open(os.path.join(ROOT, "paper_2203_09732_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
@@ -255,13 +255,13 @@ def profiled_traffic(name):
 
 
 def hv_kernel_name(L):
-    e = os.environ.get("HS_HV_SB")
-    on = (e == "1" and L >= 22) if e is not None else L >= 24
-    if not on:
-        return "k_matvec<float> (block form)"
-    if os.environ.get("HS_SB4") == "1":
-        return "k_sb4<float, MODE_HV> (four-low-bit superblock form, one lane per sub-block)"
-    return "k_sbhv<float, MODE_HV> (ten-low-bit superblock form, one warp per sub-block)"
+    if os.environ.get("HS_HV_SB") == "1" and L >= 22:
+        if os.environ.get("HS_SB4") == "1":
+            return "k_sb4<float, MODE_HV> (four-low-bit superblock form, one lane per sub-block)"
+        return "k_sbhv<float, MODE_HV> (ten-low-bit superblock form, one warp per sub-block)"
+    if L >= 24:
+        return "k_cls<MODE_HV> (one warp per block, CTAs by class)"
+    return "k_rows<float> (one thread per row)"
 
 
 def hv_roofline(torch, hs, L, stream):
@@ -734,8 +734,8 @@ def l16_batch(torch, hs, args):
 
 def forms_table(torch, hs, inputs):
     """Microseconds per product and per MINRES iteration for each row form
-    (block, ten-low-bit and four-low-bit superblock; HS_HV_SB and HS_SB4 select
-    them) at L = 24, 26, 28, FP32 and FP64, CUDA events on the current stream."""
+    (the default, ten-low-bit and four-low-bit superblock; HS_HV_SB and HS_SB4
+    select them) at L = 24, 26, 28, FP32 and FP64, CUDA events on the current stream."""
     out = {}
 
     def timed(fn, reps):
@@ -756,7 +756,7 @@ def forms_table(torch, hs, inputs):
                 for name, dt, reps in (("f32", torch.float32, 10), ("f64", torch.float64, 3)):
                     x = torch.randn(c.n, dtype=dt, device="cuda")
                     y = torch.empty_like(x)
-                    for form, env in (("block", ("0", "0")), ("sb10", ("1", "0")), ("sb4", ("1", "1"))):
+                    for form, env in (("default", ("0", "0")), ("sb10", ("1", "0")), ("sb4", ("1", "1"))):
                         os.environ["HS_HV_SB"], os.environ["HS_SB4"] = env
                         for _ in range(2):
                             c.matvec(x, y, shifted=True)

@@ -354,6 +354,17 @@ hs_status hs_create(int L, const double* h_host, double sigma, void* cuda_stream
       for (int c = 0; c < W; ++c) bt[a * W + c] = binom(a, c);
     if ((st = upload(hd, &hd->d_binom, bt)) != HS_OK) return bail(st);
   }
+  if (hd->k == KLO_MAX) {
+    // the blocks by class (hv_cls.cuh)
+    std::vector<uint32_t> order(hd->blocks.size());
+    int* first = hd->cls_first;
+    for (const BlockInfo& b : hd->blocks) ++first[b.w + 1];
+    for (int w = 0; w <= KLO_MAX; ++w) first[w + 1] += first[w];
+    int at[KLO_MAX + 1];
+    std::copy(first, first + KLO_MAX + 1, at);
+    for (size_t i = 0; i < order.size(); ++i) order[at[hd->blocks[i].w]++] = (uint32_t)i;
+    if ((st = upload(hd, &hd->d_order, order)) != HS_OK) return bail(st);
+  }
   // superblock plans for long chains; HS_SB_PLANS=1 builds them for any L
   // whose windows apply (tests of the superblock forms on small chains)
   {
@@ -382,6 +393,7 @@ void hs_free(hs_handle* hd) {
     if (hd->graph64[i]) cudaGraphExecDestroy(hd->graph64[i]);
   }
   dev_free(hd, hd->d_low);
+  dev_free(hd, hd->d_order);
   dev_free(hd, hd->d_blocks);
   dev_free(hd, hd->d_binom);
   dev_free(hd, hd->d_sigma);

@@ -27,9 +27,9 @@
 
 #include "../../include/hs.h"
 
-// hv_sb.cu: the superblock form that serves products and MINRES pass A of
-// precision dt where its plan applies: 6 or 4 low bits (sb6.cuh, sb4.cuh), or
-// ten (sb.cuh)
+// hv_sb.cu: the form of MINRES pass A and of superblock products of precision dt:
+// 6 or 4 low bits (sb6.cuh, sb4.cuh), ten (sb.cuh), or 0, the class form
+// (hv_cls.cuh) in pass A and ten in products
 int hs_want_sb(hs_dtype dt);
 
 namespace hs {
@@ -133,6 +133,8 @@ struct hs_handle {
 
   // device copies
   hs::LowEntry* d_low = nullptr;
+  uint32_t* d_order = nullptr;       // block indexes by class (k = KLO_MAX), cls_first
+  int cls_first[hs::KLO_MAX + 2] = {};
   hs::BlockInfo* d_blocks = nullptr;
   uint32_t* d_binom = nullptr;       // (LMAX + 1) x (LMAX / 2 + 2)
   double* d_sigma = nullptr;         // device copy of sigma

@@ -4,31 +4,11 @@
 #include <algorithm>
 #include <cstdlib>
 
-#include "rows.cuh"
+#include "hv_cls.cuh"
 
 namespace hs {
 
 // ---------------------------------------------------------------------------
-// y = (H - sigma * shifted) x. Warps walk the blocks in rank order. FP32 chains
-// without a superblock plan from L = 24 on.
-template <typename T>
-__global__ void __launch_bounds__(HV_THREADS) k_matvec(Geo g, const T* __restrict__ x,
-                                                       T* __restrict__ y, const double* d_sigma,
-                                                       int shifted) {
-  extern __shared__ __align__(16) char smem[];
-  const RowSmem<T> s = row_smem_setup<T>(smem, g);
-  const double sigma = shifted ? *d_sigma : 0.0;
-  const int lane = threadIdx.x & 31;
-  for_blocks(g, sigma, [&](const Hdr& h) {
-    T xi[JMAX], hx[JMAX];
-    block_hv<T>(x, s, h, xi, hx);
-    T* yb = y + h.R + lane;
-#pragma unroll
-    for (int j = 0; j < JMAX; ++j)
-      if (j < h.J && lane + 32 * j < h.C) __stcs(yb + 32 * j, hx[j]);
-  });
-}
-
 // v / 2. FP64: by the exponent where that is exact in every lane of the warp (a few
 // integer instructions instead of one on the FP64 pipe).
 __device__ __forceinline__ float half_of(float v) { return 0.5f * v; }
@@ -258,29 +238,31 @@ static hs_status prep_smem(hs_handle* hd, K kern, size_t bytes) {
 
 hs_status launch_matvec(hs_handle* hd, const void* x, void* y, hs_dtype dt, int shifted) {
   // FP64: one thread per row at every L (the six-low-bit superblock form takes
-  // 49, 137, 528 and 2084 us at L = 22 .. 28, this 35, 116, 445 and 1775). FP32:
-  // the ten-low-bit superblock form from L = 24 on (27, 82 and 333 us at L = 24,
-  // 26, 28; one thread per row 31, 123 and 600: its far gathers miss L2), and
-  // where it has no plan there the block form (36, 115, 498). HS_HV_SB=0 turns
-  // the superblock forms off, =1 uses them wherever a plan was built.
+  // 49, 137, 528 and 2084 us at L = 22 .. 28, this 35, 116, 445 and 1776). FP32:
+  // the class form from L = 24 on (22.7, 65.7 and 257 us at L = 24, 26, 28; the
+  // ten-low-bit superblock form 27, 82 and 333, one thread per row 31, 123 and
+  // 600; at L = 22 12.3 against 12.3 with one thread per row). HS_HV_SB=1 uses the
+  // superblock forms wherever a plan was built; HS_HV_CLS=0 / 1: the class form
+  // off, or wherever the blocks have ten low bits.
   const char* e = getenv("HS_HV_SB");
-  if (e ? e[0] == '1' : hd->L >= 24 && dt == HS_F32) {
+  if (e && e[0] == '1') {
     bool used = false;
     hs_status st = launch_matvec_sb(hd, x, y, dt, shifted, &used);
     if (st != HS_OK || used) return st;
   }
   const Geo g = hd->geo();
   const int nt = (*std::max_element(g.cls_C, g.cls_C + g.k + 1) + 31) / 32 * 32;
+  const char* c = getenv("HS_HV_CLS");
   if (dt == HS_F64) {
     k_rows<double><<<g.nblocks, nt, 0, hd->stream>>>(
         g, static_cast<const double*>(x), static_cast<double*>(y), hd->d_sigma, shifted);
-  } else if (hd->L < 24) {
-    k_rows<float><<<g.nblocks, nt, 0, hd->stream>>>(
-        g, static_cast<const float*>(x), static_cast<float*>(y), hd->d_sigma, shifted);
+  } else if (hd->d_order && (c ? c[0] == '1' : hd->L >= 24)) {
+    const int grid = CLS_MB * hd->num_sms;
+    k_cls<sb::MODE_HV><<<grid, CLS_NT, 0, hd->stream>>>(g, cls_work(hd, grid),
+        static_cast<const float*>(x), static_cast<float*>(y), hd->d_sigma, shifted,
+        sb::MinresArgs{});
   } else {
-    const size_t sm = smem_of<float>(hd);
-    if (prep_smem(hd, k_matvec<float>, sm) != HS_OK) return HS_CUDA;
-    k_matvec<float><<<row_grid(hd), HV_THREADS, sm, hd->stream>>>(
+    k_rows<float><<<g.nblocks, nt, 0, hd->stream>>>(
         g, static_cast<const float*>(x), static_cast<float*>(y), hd->d_sigma, shifted);
   }
   count_launches(1);

@@ -322,16 +322,17 @@ void sb_release(hs_handle* hd) {
 
 }  // namespace hs
 
-// The low bits of the superblock form: six in FP64, whose additions bound every
-// form (the six-bit one adds the fewest: no zeros for parallel mid bonds, and the
-// fewest instructions around them; L = 24: 137 us, four bits 172, block 177; L = 28:
-// 2.08 ms, 2.50, 2.64), ten in FP32, where the gathers of the whole-superblock
-// bonds bound all of them (L = 28: 334 us, six bits 344, four 392). HS_SB4=1 / 0
-// selects four or ten bits for both (tests compare forms).
+// The superblock form of MINRES pass A, and of products under HS_HV_SB=1: six low
+// bits in FP64, whose additions bound every form (no zeros for parallel mid bonds,
+// and the fewest instructions around them; a product at L = 24: 137 us, four bits
+// 172; L = 28: 2.08 ms and 2.50); in FP32 0: the class form (hv_cls.cuh; L = 28:
+// 257 us against 333 with ten bits, 344 with six, 392 with four), or ten bits
+// where it does not apply. HS_SB4=1 / 0 selects four or ten bits for both (tests
+// compare forms).
 int hs_want_sb(hs_dtype dt) {
   const char* e = getenv("HS_SB4");
   if (e) return e[0] == '1' ? 4 : 10;
-  return dt == HS_F64 ? 6 : 10;
+  return dt == HS_F64 ? 6 : 0;
 }
 
 namespace hs {

@@ -14,6 +14,7 @@
 #include "common.cuh"
 #include "minres_scalar.cuh"
 #include "sb4_kern.cuh"
+#include "hv_cls.cuh"
 #include "sb6_kern.cuh"
 #include "sb_kern.cuh"
 
@@ -80,9 +81,14 @@ hs_status solve_t(hs_handle* hd, const T* b, const MinresVecs& v, double tol, lo
   const bool use4 = want == 4 && d4 && d4->ok;
   const bool use6 = sizeof(T) == 8 && want == 6 && d6 && d6->ok;
   const auto kA6 = sb6::kernel6<double, sb::MODE_MINRES>();
-  const size_t smA = use6 ? d6->smem : use4 ? d4->smem : d->smem;
+  // FP32: the class form where the blocks have ten low bits
+  const auto kAc = k_cls<sb::MODE_MINRES>;
+  const int gc = grid_of(hd, kAc, CLS_NT, 0, CLS_MB * hd->num_sms);
+  const bool cls = sizeof(T) == 4 && want == 0 && hd->d_order && gc >= CLS_CTAS_MIN;
+  const size_t smA = cls ? 0 : use6 ? d6->smem : use4 ? d4->smem : d->smem;
   const size_t smR = sb::rows_smem_bytes<T>(1 << g.k);
-  const int gA = use6 ? grid_of(hd, kA6, sb6::NT6, smA, d6->geo.npairs)
+  const int gA = cls ? gc
+               : use6 ? grid_of(hd, kA6, sb6::NT6, smA, d6->geo.npairs)
                : use4 ? grid_of(hd, kern_A4<T>(d4->geo.km), nt_a4<T>(), smA, d4->geo.npairs)
                       : grid_of(hd, kern_A<T>(g.km), NT_A, smA, g.npairs);
   const int gI = grid_of(hd, kern_R<T, PC, sb::ROWS_INIT>(), NT_R, smR, g.npairs);
@@ -98,6 +104,7 @@ hs_status solve_t(hs_handle* hd, const T* b, const MinresVecs& v, double tol, lo
   const int gB = use_flat ? grid_of(hd, kflat, sb::NT_FLAT, 0, (int)(hd->n / 2 / sb::NT_FLAT) + 1)
                           : grid_of(hd, kern_R<T, PC, sb::ROWS_B>(), NT_R, smR, g.npairs);
   if (gA < 1 || gI < 1 || gB < 1) return HS_OK;
+  const ClsWork work = cls ? cls_work(hd, gA) : ClsWork{};
   *used = true;
   sb::MinresArgs ma;
   ma.v = v;
@@ -114,7 +121,7 @@ hs_status solve_t(hs_handle* hd, const T* b, const MinresVecs& v, double tol, lo
   // and this workspace
   cudaGraphExec_t& exec = hd->sbgraph[ti][PC];
   int* key = hd->sbgraph_key[ti][PC];
-  const int keyA = gA | (use4 ? 1 << 30 : 0) | (use6 ? 1 << 28 : 0) | (use_flat ? 1 << 29 : 0);
+  const int keyA = gA | (use4 ? 1 << 30 : 0) | (use6 ? 1 << 28 : 0) | (cls ? 1 << 27 : 0) | (use_flat ? 1 << 29 : 0);
   if (exec && (key[0] != keyA || key[1] != gB || hd->sbgraph_ws[ti] != v.q0)) {
     cudaGraphExecDestroy(exec);
     exec = nullptr;
@@ -129,7 +136,9 @@ hs_status solve_t(hs_handle* hd, const T* b, const MinresVecs& v, double tol, lo
       mA.counter = hd->d_counter + 1;
       mB.counter = hd->d_counter + 2;
       for (int it = 0; it < SB_CHUNK; ++it) {
-        if (use6)
+        if (cls)
+          kAc<<<gA, CLS_NT, 0, cs>>>(hd->geo(), work, nullptr, nullptr, hd->d_sigma, 1, mA);
+        else if (use6)
           kA6<<<gA, sb6::NT6, smA, cs>>>(d6->geo, nullptr, nullptr, hd->d_sigma, 1, mA);
         else if (use4)
           kern_A4<T>(d4->geo.km)<<<gA, nt_a4<T>(), smA, cs>>>(d4->geo, nullptr, nullptr,
