@@ -28,9 +28,10 @@ __device__ __forceinline__ double half_of(double v) {
 // and SM: 90 us), so nothing adds zeros, the low neighbours are summed by the
 // threads in the order of LowSorted (5 adds in a warp instead of 8) and the halving
 // is done on the exponent (without that and the votes on c1, c2: 119 and 469 us at
-// L = 24 and 26). k_matvec, with up to eight rows per lane, added zeros for rows and bonds that were not
-// there and copied the low table to each CTA. us, that form -> this (L = 24, 26
-// FP64: sb6 -> this; L = 24 before both 176):
+// L = 24 and 26). A form with one warp per block and up to eight rows per lane added
+// zeros for rows and bonds that were not there and copied the low table to each
+// CTA. us, that form -> this (L = 24, 26 FP64: the six-low-bit superblock form ->
+// this; L = 24 before both 176):
 //   FP64  L = 12 8.2 -> 4.1  16 10.8 -> 5.2  20 31.1 -> 14.4  22 55 -> 35  24 137 -> 116  26 528 -> 445
 //   FP32  L = 12 6.2 -> 4.1  16 6.2 -> 4.1  20 8.2 -> 6.2  22 14.4 -> 12.3
 // 40 warps per SM in FP64 (48 registers): with 32 and 48 119 and 121 us at L = 24.

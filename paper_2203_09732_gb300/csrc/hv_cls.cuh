@@ -9,8 +9,8 @@
 // order, so all warps gather from one window of x.
 // The ten-low-bit superblock form (sb_kern.cuh) issued 193 thread instructions a
 // row at L = 28 (333 us, issue 60 %); here 138, and the wavefronts of loads and
-// shared memory bound it (77 % of their peak; waits on gathers come next). us, that form -> this: L = 24 27 -> 22.7, L = 26 82 -> 65.7,
-// L = 28 333 -> 257. With the low part in registers (16 warps per SM, 228 bytes
+// shared memory bound it (77 % of their peak; waits on gathers come next). us,
+// that form -> this: L = 24 27 -> 22.7, L = 26 82 -> 65.7, L = 28 333 -> 257. With the low part in registers (16 warps per SM, 228 bytes
 // spilled) 357; with equal shares by rows 511.
 #pragma once
 #include "rows.cuh"

@@ -1,10 +1,12 @@
-// Preconditioned MINRES of Algorithm 2 (Appendix A) for long chains, on the
-// superblock layout (sb.cuh). One iteration is two launches:
-//   pass A (k_sbhv, MINRES mode): the pending d/x update of iteration k - 1,
-//          p = (H - sigma) q_k from a shared-memory tile per superblock pair,
-//          alpha_k from a last-CTA reduction;
-//   pass B (k_sbrows): q_{k+1} and beta_{k+1} with the preconditioner
-//          recomputed per row, then the Givens rotation on the device.
+// Preconditioned MINRES of Algorithm 2 (Appendix A) for long chains. One
+// iteration is two launches:
+//   pass A: p = (H - sigma) q_k and alpha_k from a last-CTA reduction. FP32: the
+//          class form (hv_cls.cuh); FP64: the six-low-bit superblock form (sb6.cuh);
+//   pass B: the d/x update of iteration k - 1, q_{k+1} and beta_{k+1}, then the
+//          Givens rotation on the device. FP32: blk_rows.cuh, M formed per row;
+//          FP64: k_flat_B, M and 1/M in memory.
+// HS_SB4 selects the ten- or four-low-bit superblock forms, whose passes also
+// serve blocks without the tables of those above (k_sbhv, k_sb4, k_sbrows).
 // The scalars never leave the device; chunks of iterations are replayed from
 // a captured CUDA graph, and the host reads the state once per replay to see
 // whether the solve has finished. Same vectors and arithmetic as minres.cu.
@@ -14,6 +16,7 @@
 #include "common.cuh"
 #include "minres_scalar.cuh"
 #include "sb4_kern.cuh"
+#include "blk_rows.cuh"
 #include "hv_cls.cuh"
 #include "sb6_kern.cuh"
 #include "sb_kern.cuh"
@@ -84,7 +87,8 @@ hs_status solve_t(hs_handle* hd, const T* b, const MinresVecs& v, double tol, lo
   // FP32: the class form where the blocks have ten low bits
   const auto kAc = k_cls<sb::MODE_MINRES>;
   const int gc = grid_of(hd, kAc, CLS_NT, 0, CLS_MB * hd->num_sms);
-  const bool cls = sizeof(T) == 4 && want == 0 && hd->d_order && gc >= CLS_CTAS_MIN;
+  const bool blk = sizeof(T) == 4 && want == 0;    // element-wise passes of blk_rows.cuh
+  const bool cls = blk && hd->d_order && gc >= CLS_CTAS_MIN;
   const size_t smA = cls ? 0 : use6 ? d6->smem : use4 ? d4->smem : d->smem;
   const size_t smR = sb::rows_smem_bytes<T>(1 << g.k);
   const int gA = cls ? gc
@@ -100,8 +104,12 @@ hs_status solve_t(hs_handle* hd, const T* b, const MinresVecs& v, double tol, lo
       dev_alloc(hd, (void**)&hd->sb_m, sizeof(double) * 2 * (size_t)hd->n) != HS_OK)
     hd->err.clear();
   const bool use_flat = flat && (!keeps_m || hd->sb_m);
+  const auto kIb = k_blk_rows<PC, sb::ROWS_INIT>;
+  const auto kBb = k_blk_rows<PC, sb::ROWS_B>;
+  const Geo gh = hd->geo();
   const auto kflat = sb::k_flat_B<keeps_m>;
-  const int gB = use_flat ? grid_of(hd, kflat, sb::NT_FLAT, 0, (int)(hd->n / 2 / sb::NT_FLAT) + 1)
+  const int gB = blk ? grid_of(hd, kBb, HV_THREADS, 0, (gh.nblocks + HV_WARPS - 1) / HV_WARPS)
+               : use_flat ? grid_of(hd, kflat, sb::NT_FLAT, 0, (int)(hd->n / 2 / sb::NT_FLAT) + 1)
                           : grid_of(hd, kern_R<T, PC, sb::ROWS_B>(), NT_R, smR, g.npairs);
   if (gA < 1 || gI < 1 || gB < 1) return HS_OK;
   const ClsWork work = cls ? cls_work(hd, gA) : ClsWork{};
@@ -112,16 +120,21 @@ hs_status solve_t(hs_handle* hd, const T* b, const MinresVecs& v, double tol, lo
   ma.partial = hd->d_partial;
   ma.m = keeps_m ? hd->sb_m : nullptr;
   ma.mi = ma.m ? hd->sb_m + hd->n : nullptr;
+  BlkRows cr{};
+  if (blk) cr = BlkRows{reinterpret_cast<const float*>(b), ma, tol, kmax, hd->d_sigma, g.dscale};
   // initial pass: q_1 = M^-1 b, beta_1, state
-  ma.counter = hd->d_counter + 0;
-  kern_R<T, PC, sb::ROWS_INIT>()<<<gI, NT_R, smR, hd->stream>>>(g, b, ma, tol, kmax, hd->d_sigma);
+  ma.counter = cr.ma.counter = hd->d_counter + 0;
+  if (blk)
+    kIb<<<gB, HV_THREADS, 0, hd->stream>>>(gh, cr);
+  else
+    kern_R<T, PC, sb::ROWS_INIT>()<<<gI, NT_R, smR, hd->stream>>>(g, b, ma, tol, kmax, hd->d_sigma);
   count_launches(1);
   HS_CUDA_TRY(hd, cudaGetLastError());
   // the chunk graph, cached per (precision, preconditioner) for these grids
   // and this workspace
   cudaGraphExec_t& exec = hd->sbgraph[ti][PC];
   int* key = hd->sbgraph_key[ti][PC];
-  const int keyA = gA | (use4 ? 1 << 30 : 0) | (use6 ? 1 << 28 : 0) | (cls ? 1 << 27 : 0) | (use_flat ? 1 << 29 : 0);
+  const int keyA = gA | (use4 ? 1 << 30 : 0) | (use6 ? 1 << 28 : 0) | (cls ? 1 << 27 : 0) | (blk ? 1 << 26 : 0) | (use_flat ? 1 << 29 : 0);
   if (exec && (key[0] != keyA || key[1] != gB || hd->sbgraph_ws[ti] != v.q0)) {
     cudaGraphExecDestroy(exec);
     exec = nullptr;
@@ -135,9 +148,12 @@ hs_status solve_t(hs_handle* hd, const T* b, const MinresVecs& v, double tol, lo
       sb::MinresArgs mA = ma, mB = ma;
       mA.counter = hd->d_counter + 1;
       mB.counter = hd->d_counter + 2;
+      BlkRows cB = cr;
+      cB.ma = mB;
+      cB.b = nullptr;
       for (int it = 0; it < SB_CHUNK; ++it) {
         if (cls)
-          kAc<<<gA, CLS_NT, 0, cs>>>(hd->geo(), work, nullptr, nullptr, hd->d_sigma, 1, mA);
+          kAc<<<gA, CLS_NT, 0, cs>>>(gh, work, nullptr, nullptr, hd->d_sigma, 1, mA);
         else if (use6)
           kA6<<<gA, sb6::NT6, smA, cs>>>(d6->geo, nullptr, nullptr, hd->d_sigma, 1, mA);
         else if (use4)
@@ -145,7 +161,9 @@ hs_status solve_t(hs_handle* hd, const T* b, const MinresVecs& v, double tol, lo
                                                               hd->d_sigma, 1, mA);
         else
           kern_A<T>(g.km)<<<gA, NT_A, smA, cs>>>(g, nullptr, nullptr, hd->d_sigma, 1, mA);
-        if (use_flat)
+        if (blk)
+          kBb<<<gB, HV_THREADS, 0, cs>>>(gh, cB);
+        else if (use_flat)
           kflat<<<gB, sb::NT_FLAT, 0, cs>>>(hd->n / 2, mB);
         else
           kern_R<T, PC, sb::ROWS_B>()<<<gB, NT_R, smR, cs>>>(g, nullptr, mB, 0.0, 0, hd->d_sigma);
