@@ -71,11 +71,12 @@ typedef struct {
 
 /* Solver forms (all run the recurrence of Algorithm 2): vectors resident on
  * chip (HS_FORM_SMEM: one thread-block cluster for chains of up to 16384 rows,
- * in FP64 up to 4096, else shared memory of the whole grid, chains up to
- * L = 20 in FP64, 22 in FP32); superblock passes
- * (from L = 24 on); one persistent cooperative kernel with vectors in global
- * memory; per-pass kernels replayed from a CUDA graph; and the shared-memory
- * form with one global reduction per iteration (the product taken of
+ * in FP64 up to 4096, else the registers or shared memory of the whole grid,
+ * chains up to L = 20 in FP64, 22 in FP32); passes on the blocks and
+ * superblocks of long chains (HS_FORM_SUPERBLOCK, from L = 24 on, in FP64 from
+ * L = 22 on); one persistent cooperative kernel with vectors in global
+ * memory; per-pass kernels replayed from a CUDA graph; and the on-chip form
+ * with one global reduction per iteration (the product taken of
  * M^-1 p_k, p carried by the recurrence of q and replaced by a product every
  * R steps, beta_{k+1}^2 expanded in sums known before alpha_k: equal in exact
  * arithmetic, different in rounding). */
@@ -146,11 +147,10 @@ hs_status hs_diag(hs_handle* hd, double* diag_dev, hs_precond pc, double* minv_d
  * FP32 (x, y float, FP32 accumulation) or FP64. x and y must not overlap and
  * must be aligned to their element size (any offset from that is fine).
  * Eq. (1); element (i, k) for i != k is 1/2 exactly when states i and k differ
- * by the flip of one antiparallel bond (Appendix C). From L = 24 on, FP32 uses
- * the superblock form (x of two superblocks staged in shared memory); the
- * environment variable HS_HV_SB=0 selects the block form, HS_HV_SB=1 the
- * superblock form for both precisions from L = 22 on. Both forms give the
- * same values up to the order of the row sums. */
+ * by the flip of one antiparallel bond (Appendix C). The environment variable
+ * HS_HV_SB=1 selects the superblock forms (x of two superblocks staged in shared
+ * memory) from L = 22 on. All forms give the same values up to the order of the
+ * row sums. */
 hs_status hs_matvec(hs_handle* hd, const void* x_dev, void* y_dev, hs_dtype dtype,
                     int shifted);
 
