@@ -14,7 +14,7 @@ from tests.test_sb_host import HERE, _nvcc
 
 
 @pytest.fixture(scope="module")
-def checker(tmp_path_factory):
+def rows_prog(tmp_path_factory):
     nvcc = _nvcc()
     if nvcc is None:
         pytest.skip("nvcc not found")
@@ -31,7 +31,7 @@ def checker(tmp_path_factory):
 @pytest.mark.parametrize("L,KS", [(10, 7), (10, 8), (12, 7), (12, 10), (14, 8), (14, 12), (16, 9),
                                   (16, 14), (18, 13), (18, 14), (20, 10), (22, 12), (24, 13),
                                   (24, 14)])
-def test_rows_vs_explicit_matrix(checker, tmp_path, L, KS):
+def test_rows_vs_explicit_matrix(rows_prog, tmp_path, L, KS):
     """Every row in FP64 (1e-14 of the row scale, as in test_sb_host.py) and FP32 (the
     rounding bound of an FP32 row sum)."""
     h = np.asarray(inputs.disorder(L, 3.0, 3 * L + KS), dtype=np.float64)
@@ -45,7 +45,7 @@ def test_rows_vs_explicit_matrix(checker, tmp_path, L, KS):
     ref32 = H @ x32 - sigma * x32
     bound32 = (L + 4) * 2.0 ** -24 * (np.abs(diag - sigma) * np.abs(x32) + abs(H) @ np.abs(x32)) * 2
     scale = np.abs(diag * x).max() + np.abs(x).max() * L
-    r = subprocess.run([checker, str(L), str(KS), repr(sigma), str(tmp_path)],
+    r = subprocess.run([rows_prog, str(L), str(KS), repr(sigma), str(tmp_path)],
                        capture_output=True, text=True)
     assert r.returncode == 0, (r.stdout, r.stderr)
     y64 = np.fromfile(tmp_path / "y64.bin")
@@ -55,11 +55,11 @@ def test_rows_vs_explicit_matrix(checker, tmp_path, L, KS):
     assert (np.abs(y32 - ref32) <= bound32 + 1e-30).all()
 
 
-def test_plan_rejects_splits_out_of_range(checker, tmp_path):
+def test_plan_rejects_splits_out_of_range(rows_prog, tmp_path):
     """No mid bit, more than 8, or fewer than two top bits: no plan."""
     L = 16
     np.asarray(inputs.disorder(L, 1.0, 1), dtype=np.float64).tofile(tmp_path / "h.bin")
     for KS in (6, 15, 16):
-        r = subprocess.run([checker, str(L), str(KS), "0.0", str(tmp_path)],
+        r = subprocess.run([rows_prog, str(L), str(KS), "0.0", str(tmp_path)],
                            capture_output=True, text=True)
         assert r.returncode == 4 and "does not apply" in r.stdout
