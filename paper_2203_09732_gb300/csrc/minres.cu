@@ -685,11 +685,12 @@ static bool force_global() {
 // cannot hold, from L = 24 on. HS_MINRES_SB=0 turns it off; =1 makes it the
 // first choice wherever a superblock plan exists (tests compare forms).
 // FP64: from L = 22 on (L = 22: 78 us per iteration, 138 in the persistent form
-// that took it before).
-static int sb_choice(const hs_handle* hd, bool f64) {
+// that took it before), but with Jacobi from L = 24 on as in FP32: its passes
+// refuse a_ii - sigma at the rounding level, which the persistent form accepts.
+static int sb_choice(const hs_handle* hd, bool f64, int pc) {
   const char* e = getenv("HS_MINRES_SB");
   if (e) return e[0] == '1' ? 2 : 0;
-  return hd->L >= (f64 ? 22 : 24) ? 1 : 0;
+  return hd->L >= (f64 && pc != 1 ? 22 : 24) ? 1 : 0;
 }
 
 // The one-reduction recurrence is the first choice for FP64 solves with the
@@ -751,7 +752,7 @@ static hs_status solve_pc(hs_handle* hd, const T* b, T* x, double tol, long long
   if (st != HS_OK) return st;
   st = HS_CUDA;
   int form = 0;
-  const int sbc = sb_choice(hd, sizeof(T) == 8);
+  const int sbc = sb_choice(hd, sizeof(T) == 8, PC);
   if (sbc == 2 && (st = try_sb<T, PC>(hd, b, v, tol, kmax)) != HS_CUDA) form = HS_FORM_SUPERBLOCK;
   const int cs = st == HS_CUDA && !force_graph() && !force_global()
                      ? cluster_choice(hd, sizeof(T) == 8, PC) : 0;

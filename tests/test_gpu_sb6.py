@@ -1,4 +1,4 @@
-"""GPU parity of the six-low-bit superblock product (FP64, the default from
+"""GPU parity of the six-low-bit superblock product (FP64 MINRES pass A from
 L = 22 on) on small chains over windows that reach every bond kind, at L = 22 and
 24 in full, and of MINRES on it (its default at L = 22)."""
 import numpy as np
@@ -7,7 +7,7 @@ import scipy.sparse as sp
 
 from oracle import hamiltonian, minres
 from paper_2203_09732_gb300 import inputs
-from tests.gpu_util import need_gpu, to_dev
+from tests.gpu_util import need_gpu, to_dev, torch
 from tests.test_gpu_minres import TOL64, separated_sigma
 
 pytestmark = pytest.mark.gpu
@@ -52,3 +52,18 @@ def test_minres_iterates_l22(kind):
             x, info = c.minres(to_dev(b), tol=0.0, kmax=k, precond=kind, allow_not_converged=True)
             assert info["iters"] == k and info["form"] == hs.FORM_SUPERBLOCK
             assert np.abs(x.cpu().numpy() - xr).max() <= TOL64[k] * np.abs(xr).max()
+
+
+def test_routes_at_l22():
+    """FP64 at L = 22: the two-pass form with the row norm; Jacobi keeps the
+    persistent form, also where a_ii - sigma is at the rounding level, which the
+    two-pass form refuses."""
+    hs = need_gpu()
+    L = 22
+    hv = inputs.disorder(L, 3.0, 0)
+    with hs.Chain(L, hv, sigma=0.0) as c:
+        c.sigma = float(c.diag()[0][12345].item()) + 1e-14
+        b = to_dev(inputs.gaussian(c.n, 3))
+        for kind, form in (("row", hs.FORM_SUPERBLOCK), ("jacobi", hs.FORM_PERSISTENT)):
+            x, info = c.minres(b, tol=0.0, kmax=3, precond=kind, allow_not_converged=True)
+            assert info["form"] == form and info["iters"] == 3 and torch.isfinite(x).all()
