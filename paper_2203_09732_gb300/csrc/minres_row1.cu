@@ -264,6 +264,7 @@ __global__ void __launch_bounds__(ONE_NT, 1) k_minres_row1(RowArgs ra, int pc, i
         sh.s[j] = tot;
         bar_arrive(j == 0 ? &sh.barQ : &sh.barS);
       }
+      __syncwarp();                              // warp 0 reads sh.s[0] in every lane
       return true;
     };
     if (j > 0) {
