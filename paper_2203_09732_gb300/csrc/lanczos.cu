@@ -10,7 +10,7 @@
 #include <vector>
 
 #include "lanczos.cuh"
-#include "minres_smem.cuh"
+#include "minres_clu.cuh"
 
 namespace hs {
 
@@ -188,7 +188,7 @@ hs_status extremal_small(const std::vector<hs_handle*>& hds, int max_steps, doub
       break;
     }
     st = launch_clu_many(reinterpret_cast<const SmemJob*>(mem), (int)jobs.size(), n, h0->L, 0, cs,
-                         h0->stream, tr, 2 * N);
+                         h0->stream, tr, 2 * N, CLU_WAIT_LIMIT);
     if (st != HS_OK) break;
     if (cudaMemcpyAsync(t.data(), tr, sizeof(double) * t.size(), cudaMemcpyDeviceToHost,
                         h0->stream) != cudaSuccess ||

@@ -568,10 +568,7 @@ hs_status solve_smem_job(hs_handle* hd, const void* b, const MinresVecs& v, hs_d
   st = one ? launch_smem1(dt, pc, hd->k, hd->device, hd->stream, job, qs, ng, hc,
                           pipe_replace_period())
            : launch_smem2(dt, pc, hd->k, hd->device, hd->stream, job, qs, ng, hc);
-  if (st != HS_OK) return st;
-  HS_CUDA_TRY(hd, cudaMemcpyAsync(hd->h_state, hd->d_state, sizeof(MinresState),
-                                  cudaMemcpyDeviceToHost, hd->stream));
-  HS_CUDA_TRY(hd, cudaStreamSynchronize(hd->stream));
+  if (st != HS_OK || (st = grid_finish(hd)) != HS_OK) return st;
   const MinresState& S = *hd->h_state;
   if (one && S.status == HS_BREAKDOWN && S.pad == PIPE_EXPANSION) return HS_CUDA;
   return HS_OK;
@@ -716,10 +713,9 @@ static bool pipe_choice(const hs_handle* hd, bool f64, int pc) {
 }
 
 // The cluster form (minres_clu.cu) takes the small solves. Not where another
-// form is asked for (HS_MINRES_PIPE), nor under HS_BARRIER_LIMIT, which limits
-// the waits of the grid forms. HS_MINRES_CLUSTER=0 turns it off.
+// form is asked for (HS_MINRES_PIPE). HS_MINRES_CLUSTER=0 turns it off.
 static int cluster_choice(const hs_handle* hd, bool f64, int pc) {
-  if (getenv("HS_MINRES_PIPE") || getenv("HS_BARRIER_LIMIT")) return 0;
+  if (getenv("HS_MINRES_PIPE")) return 0;
   // FP64 above 4096 rows: 16 SMs' FP64 pipes would bound it
   if (f64 && hd->n > CLU_F64_ROWS && pipe_choice(hd, f64, pc)) return 0;
   const int bud = hd->sm_budget.load(std::memory_order_relaxed);

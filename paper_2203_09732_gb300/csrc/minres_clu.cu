@@ -11,11 +11,11 @@ namespace hs {
 namespace {
 
 template <typename T, int RPT>
-__global__ void __launch_bounds__(CLU_NT, 1) k_minres_clu(SmemJob job, int pc) {
+__global__ void __launch_bounds__(CLU_NT, 1) k_minres_clu(SmemJob job, int pc, unsigned limit) {
   extern __shared__ __align__(16) char dyn[];
   __shared__ CluShared sh;
   clu_setup(sh);
-  CluPhase ph;
+  CluPhase ph{limit};
   clu_solve<T, RPT>(job, pc, sh, dyn, ph);
   clu_sync();   // no CTA leaves while another may still write to it
 }
@@ -23,12 +23,13 @@ __global__ void __launch_bounds__(CLU_NT, 1) k_minres_clu(SmemJob job, int pc) {
 // One FP64 solve per cluster: jobs[blockIdx.x / cs] (all of one L), the
 // Lanczos scalars in trace + cluster * tstride where trace is set.
 __global__ void __launch_bounds__(CLU_NT, 1) k_minres_clu_many(const SmemJob* jobs, int pc,
-                                                               double* trace, long long tstride) {
+                                                               double* trace, long long tstride,
+                                                               unsigned limit) {
   extern __shared__ __align__(16) char dyn[];
   __shared__ CluShared sh;
   __shared__ SmemJob sj;
   clu_setup(sh);
-  CluPhase ph;
+  CluPhase ph{limit};
   const int cs = (int)clu_size(), id = (int)blockIdx.x / cs;
   if (threadIdx.x == 0) sj = jobs[id];
   __syncthreads();
@@ -39,7 +40,7 @@ __global__ void __launch_bounds__(CLU_NT, 1) k_minres_clu_many(const SmemJob* jo
 template <typename T, int RPT>
 hs_status launch_t(hs_handle* hd, const SmemJob& job, int pc, int cs) {
   return clu_launch(k_minres_clu<T, RPT>, cs, cs, clu_bytes<T>((int)hd->n, hd->L, cs, RPT),
-                    hd->stream, job, pc)
+                    hd->stream, job, pc, clu_limit())
              ? HS_OK : HS_CUDA;
 }
 
@@ -81,6 +82,12 @@ int clu_choice(long long n, int sms) {
   return cs;
 }
 
+unsigned clu_limit() {
+  const char* e = getenv("HS_BARRIER_LIMIT");
+  return e ? (unsigned)std::min<unsigned long long>(strtoull(e, nullptr, 10), CLU_WAIT_LIMIT)
+           : CLU_WAIT_LIMIT;
+}
+
 hs_status solve_clu(hs_handle* hd, const void* b, void* x, hs_dtype dt, int pc, double tol,
                     long long kmax, int cs) {
   const SmemJob job{hd->geo(), b, x, hd->d_state, hd->sigma, tol, kmax};
@@ -94,11 +101,11 @@ hs_status solve_clu(hs_handle* hd, const void* b, void* x, hs_dtype dt, int pc, 
 }
 
 hs_status launch_clu_many(const SmemJob* jobs, int count, int n, int L, int pc, int cs,
-                          cudaStream_t s, double* trace, long long tstride) {
+                          cudaStream_t s, double* trace, long long tstride, unsigned limit) {
   const int rpt = clu_rpt(n, cs);
   if (!rpt) return HS_CUDA;
   return clu_launch(k_minres_clu_many, count * cs, cs, clu_bytes<double>(n, L, cs, rpt), s, jobs, pc,
-                    trace, tstride)
+                    trace, tstride, limit)
              ? HS_OK : HS_CUDA;
 }
 

@@ -34,7 +34,8 @@ constexpr int CLU_NT = 32 * (CLU_NW + CLU_CW);
 constexpr int CLU_SIZE_MAX = 16;                // CTAs per cluster
 constexpr int CLU_RPT_MAX = 8;                  // rows per thread
 static_assert(CLU_ROWS == CLU_SIZE_MAX * 32 * CLU_NW * CLU_RPT_MAX, "rows of the largest cluster");
-// polls of an mbarrier before a wait gives up with HS_TIMEOUT
+// polls of an mbarrier before a wait gives up with HS_TIMEOUT (HS_BARRIER_LIMIT
+// sets another number for single solves and sweeps)
 constexpr unsigned CLU_WAIT_LIMIT = 1u << 22;
 
 // Exchange words of one CTA (shared memory). What one warp hands to a later
@@ -52,7 +53,8 @@ struct CluShared {
                                                 //    1/(2 beta_k^2), 1/(2 beta_k^3), beta_k/beta_{k-1}
   double alpha[2];                              // E: alpha_k
   struct { double co[4]; int apply, stop; } d[2];   // D: cq, cd1, cd2, tau (of type T)
-  int fail;
+  int fail;                                     // a wait of this CTA gave up
+  int gave_up;                                  // a wait of any CTA did (clu_agree)
   MinresState S;                                // the solve's state (rotation warp)
 };
 
@@ -88,18 +90,17 @@ __device__ __forceinline__ void bar_arm(unsigned long long* b, unsigned bytes) {
 __device__ __forceinline__ void bar_arrive(unsigned long long* b) {
   asm volatile("mbarrier.arrive.shared.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
 }
-// Waits for the phase of the given parity; false after CLU_WAIT_LIMIT polls.
-__device__ __forceinline__ bool bar_wait(unsigned long long* b, unsigned parity) {
+// Waits for the phase of the given parity (whole warps); false in every lane
+// once any lane has polled limit times in vain.
+__device__ __forceinline__ bool bar_wait(unsigned long long* b, unsigned parity, unsigned limit) {
   const uint32_t a = smem_u32(b);
-  for (unsigned it = 0; it < CLU_WAIT_LIMIT; ++it) {
-    uint32_t done;
+  uint32_t done = 0;
+  for (unsigned it = 0; it < limit && !done; ++it)
     asm volatile("{\n.reg .pred p;\n"
                  "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
                  "selp.u32 %0, 1, 0, p;\n}"
                  : "=r"(done) : "r"(a), "r"(parity) : "memory");
-    if (done) return true;
-  }
-  return false;
+  return __all_sync(0xffffffffu, done);
 }
 // One or two values into another CTA's shared memory, counted by its mbarrier.
 __device__ __forceinline__ void clu_send(uint32_t dst, double v, uint32_t bar) {
@@ -140,8 +141,10 @@ __host__ __device__ inline size_t clu_bytes(int n, int L, int cs, int rpt) {
   return clu_q_bytes<T>(n, cs, rpt) + sizeof(uint32_t) * (size_t)(L / 2) * 32 * CLU_NW * rpt;
 }
 
-// Phase parities of a cluster's barriers, carried from solve to solve.
+// Phase parities of a cluster's barriers, carried from solve to solve, and the
+// polls of a wait.
 struct CluPhase {
+  unsigned limit;
   unsigned a = 0, b = 0, c = 0, d[2] = {0, 0}, e[2] = {0, 0}, f[2] = {0, 0};
 };
 
@@ -156,11 +159,28 @@ __device__ __forceinline__ void clu_setup(CluShared& sh) {
       bar_init(&sh.barE[i], 1);
       bar_init(&sh.barD[i], 1);
     }
-    sh.fail = 0;
+    sh.fail = sh.gave_up = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
   clu_sync();
+}
+
+// Whether a wait of any CTA of the cluster gave up, the same answer in all of
+// them (all threads, after a CTA barrier behind the last write of sh.fail). If
+// so, messages sent to a CTA that stopped waiting may still be under way: every
+// CTA waits a while after all have stopped sending, so that none leaves before
+// they have landed, and the barriers are out of step: no solve may follow.
+__device__ __forceinline__ bool clu_agree(CluShared& sh) {
+  if (sh.fail && threadIdx.x < clu_size())
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(
+                     clu_map(smem_u32(&sh.gave_up), threadIdx.x)), "r"(1) : "memory");
+  __syncwarp();
+  clu_sync();
+  if (sh.gave_up == 0) return true;
+  for (int i = 0; i < 100; ++i) __nanosleep(1000);
+  clu_sync();
+  return false;
 }
 
 // Sum of the np partials of all warps of the cluster, in every lane.
@@ -316,8 +336,8 @@ __device__ __forceinline__ void clu_row(const Geo& g, uint32_t i, int lo, int hi
 // job. Where trace is set, CTA 0 writes alpha_k to trace[2 (k - 1)] and beta_{k+1}
 // to trace[2 (k - 1) + 1] (k = 1 .. kmax): the tridiagonal matrix of the Lanczos
 // process that MINRES runs on. Rows are dealt to the CTAs in contiguous runs of rank order. Returns
-// false when a wait gave up (status HS_TIMEOUT). The final state is in sh.S of
-// every CTA and, if job.st is set, in *job.st.
+// false in every CTA when a wait of any gave up (status HS_TIMEOUT). The final state
+// is in sh.S of every CTA and, if job.st is set, in *job.st.
 //
 // Order of events (k = 1, 2, ...; the phases of a barrier follow each other
 // because each is complete only when every warp of the cluster has sent, and a
@@ -356,7 +376,7 @@ __device__ bool clu_solve(const SmemJob& job, int pc, CluShared& sh, char* dyn, 
   auto take = [&](unsigned long long* bar, unsigned bytes, unsigned& parity) {
     if (lane == 0) bar_arm(bar, bytes);
     __syncwarp();
-    const bool got = bar_wait(bar, parity);
+    const bool got = bar_wait(bar, parity, ph.limit);
     parity ^= 1u;
     return got;
   };
@@ -428,12 +448,12 @@ __device__ bool clu_solve(const SmemJob& job, int pc, CluShared& sh, char* dyn, 
     zm = warp_sum_all(zm);
     if (lane < cs) clu_send(clu_map(aSA, lane), zm, clu_map(aBarA, lane));
     // step 0 of D: the initial state
-    bool ok = bar_wait(&sh.barD[0], ph.d[0]);
+    bool ok = bar_wait(&sh.barD[0], ph.d[0], ph.limit);
     ph.d[0] ^= 1u;
     bool run = ok && sh.d[0].stop == 0;
     unsigned pb = ph.b;
     for (int k = 1; run; ++k) {
-      if (!(ok = bar_wait(&sh.barB, pb))) break;   // q_k has arrived
+      if (!(ok = bar_wait(&sh.barB, pb, ph.limit))) break;   // q_k has arrived
       pb ^= 1u;
       // p_k, doubled: 2 (H - sigma) q = (2 a_ii - 2 sigma) q_i + sum over neighbours
       T p[RPT];
@@ -456,7 +476,7 @@ __device__ bool clu_solve(const SmemJob& job, int pc, CluShared& sh, char* dyn, 
       // d_{k-2} and x_{k-2} while alpha_k travels
       if (k > 2) {
         const int t = k & 1;
-        if (!(ok = bar_wait(&sh.barD[t], ph.d[t]))) break;
+        if (!(ok = bar_wait(&sh.barD[t], ph.d[t], ph.limit))) break;
         ph.d[t] ^= 1u;
         if (sh.d[t].apply) {
           const T* co = reinterpret_cast<const T*>(sh.d[t].co);
@@ -471,7 +491,7 @@ __device__ bool clu_solve(const SmemJob& job, int pc, CluShared& sh, char* dyn, 
         }
         if (sh.d[t].stop) break;
       }
-      if (!(ok = bar_wait(&sh.barC, ph.c))) break;
+      if (!(ok = bar_wait(&sh.barC, ph.c, ph.limit))) break;
       ph.c ^= 1u;
       const T* co = reinterpret_cast<const T*>(sh.c);
       const T c1 = co[0], c2 = co[1], c3 = co[2];
@@ -518,7 +538,7 @@ __device__ bool clu_solve(const SmemJob& job, int pc, CluShared& sh, char* dyn, 
       // state) says stop
       if (k == 1 || k > 2) {
         const int v = k == 1 ? 0 : t;
-        if (!(ok = bar_wait(&sh.barD[v], ph.d[v]))) break;
+        if (!(ok = bar_wait(&sh.barD[v], ph.d[v], ph.limit))) break;
         ph.d[v] ^= 1u;
         if (sh.d[v].stop) break;
       }
@@ -531,18 +551,18 @@ __device__ bool clu_solve(const SmemJob& job, int pc, CluShared& sh, char* dyn, 
       const int t = k & 1;
       if (!(ok = take(&sh.barA, bytesA, ph.a))) break;
       if (k > 0) {
-        if (!(ok = bar_wait(&sh.barF[t], ph.f[t]))) break;
+        if (!(ok = bar_wait(&sh.barF[t], ph.f[t], ph.limit))) break;
         ph.f[t] ^= 1u;
       }
       if (k > 2) {
-        if (!(ok = bar_wait(&sh.barD[t], ph.d[t]))) break;
+        if (!(ok = bar_wait(&sh.barD[t], ph.d[t], ph.limit))) break;
         ph.d[t] ^= 1u;
         if (sh.d[t].stop) break;
       }
       const double tot = clu_total(sh.slotA, np);
       if (k == 0) {
         if (lane == 0) { sh.alpha[0] = tot; bar_arrive(&sh.barE[0]); }
-        if (!(ok = bar_wait(&sh.barD[0], ph.d[0]))) break;
+        if (!(ok = bar_wait(&sh.barD[0], ph.d[0], ph.limit))) break;
         ph.d[0] ^= 1u;
         if (sh.d[0].stop) {                      // beta_1 came, but no product follows
           ph.f[1] ^= 1u;
@@ -564,12 +584,13 @@ __device__ bool clu_solve(const SmemJob& job, int pc, CluShared& sh, char* dyn, 
   } else if (wid == 1 - CLU_CW) {
     // ---- rotation warp: step k - 1 in iteration k (k = 1: the initial state)
     MinresState S{};
+    S.k = 1;
     bool ok = true;
     for (int k = 1;; ++k) {
       const int t = k & 1, u = t ^ 1;
-      if (!(ok = bar_wait(&sh.barF[t], ph.f[t]))) break;
+      if (!(ok = bar_wait(&sh.barF[t], ph.f[t], ph.limit))) break;
       ph.f[t] ^= 1u;
-      if (!(ok = bar_wait(&sh.barE[u], ph.e[u]))) break;
+      if (!(ok = bar_wait(&sh.barE[u], ph.e[u], ph.limit))) break;
       ph.e[u] ^= 1u;
       if (S.done != 0) break;                    // an iteration begun past the last step
       const double al = sh.alpha[u];
@@ -589,16 +610,19 @@ __device__ bool clu_solve(const SmemJob& job, int pc, CluShared& sh, char* dyn, 
       }
       if (S.done != 0 && k == 1) break;
     }
-    if (!ok) { sh.fail = 1; S.status = HS_TIMEOUT; }
+    if (!ok) sh.fail = 1;
     S.pending = 0;
     S.done = 2;
-    if (lane == 0) {
-      sh.S = S;
-      if (me == 0 && job.st) *job.st = S;
-    }
+    if (lane == 0) sh.S = S;
   }
   __syncthreads();
-  return sh.fail == 0;
+  const bool ok = clu_agree(sh);
+  if (threadIdx.x == 0) {
+    if (!ok) sh.S.status = HS_TIMEOUT;
+    if (me == 0 && job.st) *job.st = sh.S;
+  }
+  __syncthreads();
+  return ok;
 }
 
 // The rows per thread that a chain of n rows needs on cs CTAs; 0: too many.

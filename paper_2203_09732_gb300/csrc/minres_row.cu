@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(ROW_NT, 1) k_minres_row(RowArgs ra, int pc) {
       }
       send(sh.partB, &sh.barB, acc);
     }
-    if (!ok) sh.fail = 1;
+    if (!ok) row_fail(sh.fail, ra.err);
     T* xo = reinterpret_cast<T*>(job.x);
 #pragma unroll
     for (int j = 0; j < RPT; ++j)
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(ROW_NT, 1) k_minres_row(RowArgs ra, int pc) {
         if (sh.d[v].stop) break;
       }
     }
-    if (!ok) sh.fail = 1;
+    if (!ok) row_fail(sh.fail, ra.err);
   } else if (wid == -CLU_CW) {
     // ---- alpha warp
     bool ok = true;
@@ -280,10 +280,11 @@ __global__ void __launch_bounds__(ROW_NT, 1) k_minres_row(RowArgs ra, int pc) {
       }
       if (lane == 1) { sh.alpha[t] = al; bar_arrive(&sh.barE[t]); }
     }
-    if (!ok) sh.fail = 1;
+    if (!ok) row_fail(sh.fail, ra.err);
   } else if (wid == 1 - CLU_CW) {
     // ---- rotation warp
     MinresState S{};
+    S.k = 1;
     bool ok = true;
     unsigned pf[2] = {0, 0}, pe[2] = {0, 0};
     for (int k = 1;; ++k) {
@@ -310,7 +311,7 @@ __global__ void __launch_bounds__(ROW_NT, 1) k_minres_row(RowArgs ra, int pc) {
       }
       if (S.done != 0 && k == 1) break;
     }
-    if (!ok) sh.fail = 1;
+    if (!ok) row_fail(sh.fail, ra.err);
     S.pending = 0;
     S.done = 2;
     if (!ok) S.status = HS_TIMEOUT;
@@ -375,10 +376,14 @@ hs_status row_args(hs_handle* hd, const void* b, const MinresVecs& v, double tol
   return HS_OK;
 }
 
-hs_status row_finish(hs_handle* hd) {
+hs_status grid_finish(hs_handle* hd) {
+  int* gave_up = reinterpret_cast<int*>(hd->h_pinned);
   HS_CUDA_TRY(hd, cudaMemcpyAsync(hd->h_state, hd->d_state, sizeof(MinresState),
                                   cudaMemcpyDeviceToHost, hd->stream));
+  HS_CUDA_TRY(hd, cudaMemcpyAsync(gave_up, hd->d_counter + 10, sizeof(int), cudaMemcpyDeviceToHost,
+                                  hd->stream));
   HS_CUDA_TRY(hd, cudaStreamSynchronize(hd->stream));
+  if (*gave_up) hd->h_state->status = HS_TIMEOUT;
   return HS_OK;
 }
 
@@ -389,7 +394,7 @@ hs_status solve_row(hs_handle* hd, const void* b, const MinresVecs& v, hs_dtype 
   hs_status st = row_args(hd, b, v, tol, kmax, 2, &ra, &G);
   if (st != HS_OK) return st;
   st = dt == HS_F64 ? launch_row<double>(hd, ra, pc, G) : launch_row<float>(hd, ra, pc, G);
-  return st != HS_OK ? st : row_finish(hd);
+  return st != HS_OK ? st : grid_finish(hd);
 }
 
 }  // namespace hs

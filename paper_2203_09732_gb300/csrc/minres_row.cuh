@@ -18,19 +18,27 @@ struct RowArgs {
   void* w1;
 };
 
-// Wait for a barrier of this CTA; false once a warp has set fail.
+// Wait for a barrier of this CTA (whole warps); false in every lane once a warp has
+// set fail.
 __device__ __forceinline__ bool row_wait(int& fail, unsigned long long* b, unsigned parity) {
   const uint32_t a = smem_u32(b);
-  for (unsigned it = 0; it < CLU_WAIT_LIMIT; ++it) {
-    uint32_t done;
+  uint32_t done = 0;
+  for (unsigned it = 0; it < CLU_WAIT_LIMIT && !done; ++it) {
     asm volatile("{\n.reg .pred p;\n"
                  "mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2;\n"
                  "selp.u32 %0, 1, 0, p;\n}"
                  : "=r"(done) : "r"(a), "r"(parity) : "memory");
-    if (done) return true;
-    if ((it & 15u) == 15u && *(volatile int*)&fail) return false;
+    if ((it & 15u) == 15u && !done && *(volatile int*)&fail) break;
   }
-  return false;
+  return __all_sync(0xffffffffu, done);
+}
+
+// A wait of this warp gave up: the CTA's other warps stop waiting, and the host
+// reports HS_TIMEOUT whatever the state says (grid_finish): its writer may have
+// been past its own last wait.
+__device__ __forceinline__ void row_fail(int& fail, int* err) {
+  fail = 1;
+  if ((threadIdx.x & 31) == 0) atomicExch(err, 1);
 }
 
 // Deals rows r0 .. r0 + rows - 1 (all threads): order = their places sorted by
@@ -71,12 +79,10 @@ __device__ __forceinline__ void row_deal(const Geo& g, int r0, int rows, uint16_
 
 // Host side (minres_row.cu): the arguments of a solve on the handle's SMs with
 // its exchange words cleared; a cooperative launch (HS_CUDA without a message
-// when it does not fit or is refused; fixed: static shared memory); the state
-// into hd->h_state.
+// when it does not fit or is refused; fixed: static shared memory).
 hs_status row_args(hs_handle* hd, const void* b, const MinresVecs& v, double tol, long long kmax,
                    int exchanges, RowArgs* ra, int* G);
 hs_status row_launch(hs_handle* hd, const void* kern, int G, int nt, size_t smem, size_t fixed,
                      void** args);
-hs_status row_finish(hs_handle* hd);
 
 }  // namespace hs

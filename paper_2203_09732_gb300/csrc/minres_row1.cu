@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(ONE_NT, 1) k_minres_row1(RowArgs ra, int pc, i
         send(a);
       }
     }
-    if (!ok) sh.fail = 1;
+    if (!ok) row_fail(sh.fail, ra.err);
     T* xo = reinterpret_cast<T*>(job.x);
 #pragma unroll
     for (int j = 0; j < RPT; ++j)
@@ -278,6 +278,7 @@ __global__ void __launch_bounds__(ONE_NT, 1) k_minres_row1(RowArgs ra, int pc, i
       }
     } else {
       MinresState S{};
+      S.k = 1;
       double ib = 0.0, ibp = 1.0, S6 = 0.0;
       auto others = [&]() {
         const bool got = row_wait(sh.fail, &sh.barS, ps);
@@ -327,7 +328,7 @@ __global__ void __launch_bounds__(ONE_NT, 1) k_minres_row1(RowArgs ra, int pc, i
       if (!ok) S.status = HS_TIMEOUT;
       if (lane == 0 && cta == 0) *job.st = S;
     }
-    if (!ok) sh.fail = 1;
+    if (!ok) row_fail(sh.fail, ra.err);
   }
 }
 
@@ -365,7 +366,7 @@ hs_status solve_row1(hs_handle* hd, const void* b, const MinresVecs& v, hs_dtype
   const int r = pipe_replace_period();
   st = dt == HS_F64 ? launch_rpt<double>(hd, ra, pc, G, r) : launch_rpt<float>(hd, ra, pc, G, r);
   if (st != HS_OK) return st;
-  if ((st = row_finish(hd)) != HS_OK) return st;
+  if ((st = grid_finish(hd)) != HS_OK) return st;
   const MinresState& S = *hd->h_state;
   *broke = S.status == HS_BREAKDOWN && S.pad == PIPE_EXPANSION;
   return *broke ? HS_CUDA : HS_OK;

@@ -184,7 +184,7 @@ __device__ __forceinline__ bool slot_reduce_w0(Slot* slots, int G, int cta, unsi
     for (int q = 0; q < 8; ++q) mine = mine && (gv[q] == gen);
     if (__all_sync(0xffffffffu, mine)) break;
     if (++it > limit) { ok = 0; if (lane == 0) atomicExch(err, 1); break; }
-    if ((it & 255ull) == 0 && ld_relaxed_i32(err)) { ok = 0; break; }
+    if ((it & 255ull) == 0 && __any_sync(0xffffffffu, ld_relaxed_i32(err))) { ok = 0; break; }
   }
   asm volatile("fence.acq_rel.gpu;" ::: "memory");
   double a0 = 0.0, a1 = 0.0;
@@ -322,7 +322,7 @@ __device__ __forceinline__ bool grid_total(GridWord* slots, int G, int cta, unsi
       }
       if (__all_sync(0xffffffffu, all)) break;
       if (++it > limit) { ok = 0; if (lane == 0) atomicExch(err, 1); break; }
-      if ((it & 255ull) == 0 && ld_relaxed_i32(err)) { ok = 0; break; }
+      if ((it & 255ull) == 0 && __any_sync(0xffffffffu, ld_relaxed_i32(err))) { ok = 0; break; }
     }
     ok = __all_sync(0xffffffffu, ok);
     if (ok) {
@@ -342,7 +342,7 @@ __device__ __forceinline__ bool grid_total(GridWord* slots, int G, int cta, unsi
       tot = word_load<ORD>(slots + G + 2 * cta, g);
       if (__all_sync(0xffffffffu, g == gen)) break;
       if (++it > limit) { ok = 0; if (lane == 0) atomicExch(err, 1); break; }
-      if ((it & 255ull) == 0 && ld_relaxed_i32(err)) { ok = 0; break; }
+      if ((it & 255ull) == 0 && __any_sync(0xffffffffu, ld_relaxed_i32(err))) { ok = 0; break; }
     }
     ok = __all_sync(0xffffffffu, ok);
   }
@@ -744,9 +744,14 @@ hs_status solve_clu(hs_handle* hd, const void* b, void* x, hs_dtype dt, int pc, 
                     long long kmax, int cs);
 // FP64 solves of one chain length, one per cluster: jobs[0..count) (device);
 // trace (device, may be null): the alpha_k, beta_{k+1} of job j at trace +
-// j tstride. Asynchronous.
+// j tstride; limit: polls of a wait (clu_limit: HS_BARRIER_LIMIT or the default).
+// Asynchronous.
+unsigned clu_limit();
 hs_status launch_clu_many(const SmemJob* jobs, int count, int n, int L, int pc, int cs,
-                          cudaStream_t s, double* trace, long long tstride);
+                          cudaStream_t s, double* trace, long long tstride, unsigned limit);
+// minres_row.cu: the end of a solve on the grid: the state into hd->h_state, with
+// HS_TIMEOUT where a wait of any CTA gave up (d_counter + 10).
+hs_status grid_finish(hs_handle* hd);
 // minres_row.cu: the row form (one solve on the handle's SMs, x in v.x, the
 // state in hd->h_state); HS_CUDA without a message when it does not apply.
 hs_status solve_row(hs_handle* hd, const void* b, const MinresVecs& v, hs_dtype dt, int pc,

@@ -340,7 +340,7 @@ __device__ __forceinline__ bool grp_reduce_vec(const Grp2<double>& c, double* vb
       for (int cc = lane; cc < c.G; cc += 32) all = all && ld_relaxed_u32(vgen + (size_t)par * c.G + cc) == vg;
       if (__all_sync(0xffffffffu, all)) break;
       if (++it > c.q->limit) { ok = 0; if (lane == 0) atomicExch(c.q->err, 1); break; }
-      if ((it & 255ull) == 0 && ld_relaxed_i32(c.q->err)) { ok = 0; break; }
+      if ((it & 255ull) == 0 && __any_sync(0xffffffffu, ld_relaxed_i32(c.q->err))) { ok = 0; break; }
     }
     asm volatile("fence.acq_rel.gpu;" ::: "memory");
     ok = __all_sync(0xffffffffu, ok);
@@ -623,11 +623,11 @@ __device__ __forceinline__ double clu_sum(CluSweepShared& sh, double v, int& tur
 
 __global__ void __launch_bounds__(CLU_NT, 1) k_sweep_clu(const SweepReal* reals, int count, int* head,
                                                          int K, double tol, double minres_tol,
-                                                         int pc) {
+                                                         int pc, unsigned limit) {
   extern __shared__ __align__(16) char dyn[];
   __shared__ CluSweepShared sh;
   clu_setup(sh.clu);
-  CluPhase ph;
+  CluPhase ph{limit};
   const int cs = (int)clu_size(), me = (int)clu_rank();
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr int NT = CLU_NT;
@@ -761,7 +761,7 @@ __global__ void __launch_bounds__(CLU_NT, 1) k_sweep_clu(const SweepReal* reals,
       *sr.iters = iters;
     }
     __syncthreads();
-    if (status == HS_TIMEOUT) break;             // the barriers are out of step
+    if (status == HS_TIMEOUT) break;             // in every CTA (clu_agree)
   }
   clu_sync();
 }
@@ -811,7 +811,9 @@ hs_status tune_clu(const LzRun& r, int pc, int num_sms, cudaStream_t s, Tune* ou
       float ms = 0.f;
       for (int rep = 0; rep < 2; ++rep) {        // the first one loads the kernel
         cudaEventRecord(e0, s);
-        if (launch_clu_many(jobs, groups, (int)hd->n, hd->L, pc, cs, s, nullptr, 0) != HS_OK) break;
+        if (launch_clu_many(jobs, groups, (int)hd->n, hd->L, pc, cs, s, nullptr, 0,
+                            CLU_WAIT_LIMIT) != HS_OK)
+          break;
         cudaEventRecord(e1, s);
         if (cudaStreamSynchronize(s) != cudaSuccess) break;
         cudaEventElapsedTime(&ms, e0, e1);
@@ -1122,7 +1124,7 @@ extern "C" hs_status hs_sweep(int B, const int* L_host, const double* h_host, in
     if (cs > 0 &&
         clu_launch(k_sweep_clu, groups * cs, cs, sm, s,
                    reinterpret_cast<const SweepReal*>(cmem + ab_bytes + it_bytes + res_bytes + 16), B,
-                   chead, K, tol, minres_tol, (int)pc))
+                   chead, K, tol, minres_tol, (int)pc, clu_limit()))
       ls = HS_OK;
   }
   for (int attempt = 0; !clu && attempt < 64 && ls == HS_CUDA; ++attempt) {
