@@ -330,7 +330,11 @@ __device__ __forceinline__ bool grid_total(GridWord* slots, int G, int cta, unsi
 #pragma unroll
       for (int i = 1; i < 8; ++i)
         if (32 * i < G) s += v[i];
-      if (ORD) asm volatile("fence.acq_rel.gpu;" ::: "memory");
+      // a lane answers for words that other lanes read
+      if (ORD) {
+        asm volatile("fence.acq_rel.gpu;" ::: "memory");
+        __syncwarp();
+      }
       tot = warp_sum_all(s);
       for (int c = lane; c < G; c += 32)
         if (c > 0) word_store<false>(slots + G + 2 * c, tot, gen);
