@@ -195,6 +195,18 @@ __device__ __forceinline__ double clu_total(const double* slot, int np) {
 }
 static_assert(CLU_SIZE_MAX * CLU_NW <= 64, "clu_total adds two partials per lane");
 
+// alpha_k = q_k . p_k / beta_k^2 in odd lanes, alpha_k / beta_k in even ones, from
+// q_k . p_k (doubled) and the words of F. 1 / (2 beta_k^3) leaves the range of
+// doubles where beta_k is beyond 1e102 or below 1e-103 (a right-hand side that
+// large or small; H that large): from 2^+-330 on the quotient takes two steps.
+__device__ __forceinline__ double clu_alpha(const double* f, double qp2) {
+  const bool odd = threadIdx.x & 1;
+  const double ib = f[3];
+  const bool wide = ((unsigned)__double2hiint(ib) >> 20) - (1023u - 330u) > 660u;
+  const double a = qp2 * f[odd || wide ? 4 : 5];
+  return wide && !odd ? a * ib : a;
+}
+
 // The Givens rotation of step k (Algorithm 2) and its d/x coefficients: the
 // quantities of givens_fast, with a reciprocal square root instead of a root
 // and divisions, and one lane per scalar where the operation is the same
@@ -570,8 +582,7 @@ __device__ bool clu_solve(const SmemJob& job, int pc, CluShared& sh, char* dyn, 
         }
         continue;
       }
-      // c2 = alpha_k / beta_k, alpha_k = q.p / beta_k^2 (p doubled)
-      const double al = tot * sh.f[t][lane & 1 ? 4 : 5];
+      const double al = clu_alpha(sh.f[t], tot);
       if (lane == 0) {
         T* co = reinterpret_cast<T*>(sh.c);
         co[0] = (T)sh.f[t][3]; co[1] = (T)al; co[2] = (T)sh.f[t][6];
