@@ -10,7 +10,7 @@
 #include <vector>
 
 #include "lanczos.cuh"
-#include "minres_clu.cuh"
+#include "minres_smem.cuh"
 
 namespace hs {
 
@@ -148,9 +148,10 @@ void tridiag_extremes(const double* a, const double* b, int k, double* lo, doubl
 // with the identity preconditioner and no shift, so one launch of that kernel
 // with its scalars traced gives T of N steps for every handle; the ends of T_N
 // and T_{N-10} are compared on the host, and N doubles where they still move.
-// One launch and one copy per attempt instead of nine launches and two host
+// One launch and two copies per attempt instead of nine launches and two host
 // round trips per step (n = 924: 5.4 -> 0.38 ms). HS_CUDA without a message: not
-// applicable.
+// applicable, or a run did not end well (a wait that gave up, a sum beyond the
+// range of doubles, T singular to the last bit): the plain recurrence decides.
 hs_status extremal_small(const std::vector<hs_handle*>& hds, int max_steps, double tol, double* emin,
                          double* emax) {
   hs_handle* h0 = hds[0];
@@ -162,12 +163,14 @@ hs_status extremal_small(const std::vector<hs_handle*>& hds, int max_steps, doub
   const size_t vb = (sizeof(double) * n + 255) & ~(size_t)255;
   const size_t tb = sizeof(double) * 2 * (size_t)max_steps * cnt;
   char* mem = nullptr;
-  hs_status st = dev_alloc(h0, (void**)&mem, jb + vb + tb);
+  hs_status st = dev_alloc(h0, (void**)&mem, jb + vb + tb + sizeof(MinresState) * cnt);
   if (st != HS_OK) return st;
   double* v = reinterpret_cast<double*>(mem + jb);
   double* tr = reinterpret_cast<double*>(mem + jb + vb);
+  MinresState* states = reinterpret_cast<MinresState*>(mem + jb + vb + tb);
   st = vsplitmix(h0, 0x5EEDULL, v, n);
   std::vector<double> t;
+  std::vector<MinresState> end(cnt);
   std::vector<char> todo(cnt, 1);
   int left = cnt;
   for (int N = std::min(96, max_steps); st == HS_OK && left; N = std::min(2 * N, max_steps)) {
@@ -175,7 +178,7 @@ hs_status extremal_small(const std::vector<hs_handle*>& hds, int max_steps, doub
     std::vector<int> who;
     for (int i = 0; i < cnt; ++i)
       if (todo[i]) {
-        jobs.push_back(SmemJob{hds[i]->geo(), v, nullptr, nullptr, 0.0, 0.0, N});
+        jobs.push_back(SmemJob{hds[i]->geo(), v, nullptr, states + jobs.size(), 0.0, 0.0, N});
         who.push_back(i);
       }
     t.assign((size_t)2 * N * jobs.size(), 0.0);
@@ -188,16 +191,19 @@ hs_status extremal_small(const std::vector<hs_handle*>& hds, int max_steps, doub
       break;
     }
     st = launch_clu_many(reinterpret_cast<const SmemJob*>(mem), (int)jobs.size(), n, h0->L, 0, cs,
-                         h0->stream, tr, 2 * N, CLU_WAIT_LIMIT);
+                         h0->stream, tr, 2 * N, clu_limit());
     if (st != HS_OK) break;
     if (cudaMemcpyAsync(t.data(), tr, sizeof(double) * t.size(), cudaMemcpyDeviceToHost,
                         h0->stream) != cudaSuccess ||
+        cudaMemcpyAsync(end.data(), states, sizeof(MinresState) * jobs.size(),
+                        cudaMemcpyDeviceToHost, h0->stream) != cudaSuccess ||
         cudaStreamSynchronize(h0->stream) != cudaSuccess) {
       cudaGetLastError();
       st = fail(h0, HS_CUDA, "hs_extremal: Lanczos run failed");
       break;
     }
     for (size_t w = 0; w < who.size(); ++w) {
+      if (end[w].status != HS_OK) { st = HS_CUDA; break; }
       const double* p = &t[2 * (size_t)N * w];
       std::vector<double> a, b;
       bool ended = false;                            // the Krylov space ran out
