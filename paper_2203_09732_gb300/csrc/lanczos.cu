@@ -156,7 +156,13 @@ hs_status extremal_small(const std::vector<hs_handle*>& hds, int max_steps, doub
                          double* emax) {
   hs_handle* h0 = hds[0];
   const int n = (int)h0->n, cnt = (int)hds.size();
-  const int cs = n <= CLU_F64_ROWS ? clu_choice(n, h0->num_sms) : 0;
+  // clusters no larger than the SM share of any of the handles
+  int sms = h0->num_sms;
+  for (const hs_handle* hd : hds) {
+    const int bud = hd->sm_budget.load(std::memory_order_relaxed);
+    if (bud > 0) sms = std::min(sms, bud);
+  }
+  const int cs = n <= CLU_F64_ROWS ? clu_choice(n, sms) : 0;
   if (cs < 1) return HS_CUDA;
   max_steps = std::min(max_steps, n);
   const size_t jb = (sizeof(SmemJob) * cnt + 255) & ~(size_t)255;

@@ -36,3 +36,17 @@ def test_extremes_under_a_wait_limit(L, monkeypatch):
         emin, emax, mid = c.extremal()
         assert max(abs(emin - w[0]), abs(emax - w[-1])) <= 1e-10 * (w[-1] - w[0])
         assert abs(c.sigma - 0.5 * (w[0] + w[-1])) <= 1e-10 * (w[-1] - w[0])
+
+
+@pytest.mark.parametrize("nsm", [1, 3, 0])
+def test_extremes_within_an_sm_share(nsm):
+    """The extremes with the handle held to a share of the SMs (at L = 14 a cluster
+    of one or two CTAs cannot hold the rows, and the plain recurrence runs)."""
+    hs = need_gpu()
+    for L in (8, 12, 14):
+        hv = inputs.disorder(L, 3.0, 4)
+        with hs.Chain(L, hv, sigma=0.0) as c:
+            ref = c.extremal()
+            c.set_sm_budget(nsm)
+            got = c.extremal()
+        assert max(abs(a - b) for a, b in zip(got, ref)) <= 1e-10 * (ref[1] - ref[0])
