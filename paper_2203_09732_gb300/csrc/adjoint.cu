@@ -105,9 +105,7 @@ __global__ void __launch_bounds__(HV_THREADS) k_site_sums(Geo g, const uint32_t*
 // out[j] = sum_a a_a b_a s_j(a) with s_j = +-1/2 (j < L), out[L] = sum_a a_a b_a.
 hs_status site_sums(hs_handle* hd, const double* a, const double* b, double* out) {
   const size_t sm = row_smem_bytes<double>((int)hd->low.size());
-  if (sm > 48 * 1024)
-    HS_CUDA_TRY(hd, cudaFuncSetAttribute(k_site_sums, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sm));
+  if (!allow_smem(k_site_sums, sm)) return fail(hd, HS_CUDA, "hs_twist_grad: shared memory");
   const int grid = row_grid(hd);
   k_site_sums<<<grid, HV_THREADS, sm, hd->stream>>>(hd->geo(), hd->d_binom, a, b, hd->d_partial);
   count_launches(1);
@@ -174,10 +172,7 @@ extern "C" hs_status hs_twist_grad(hs_handle* hd, const double* psi_dev, const d
     double zz[2];
     if ((st = launch_twist(hd, u, 1, zz)) != HS_OK) break;
     if (z_host) { z_host[2 * q] = zz[0]; z_host[2 * q + 1] = zz[1]; }
-    if (sm > 48 * 1024 &&
-        cudaFuncSetAttribute(k_twist_weight, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) !=
-            cudaSuccess) {
-      cudaGetLastError();
+    if (!allow_smem(k_twist_weight, sm)) {
       st = fail(hd, HS_CUDA, "hs_twist_grad: shared memory");
       break;
     }

@@ -64,6 +64,19 @@ void dev_free(hs_handle* hd, void* p) {
   else cudaFree(p);
 }
 
+bool allow_smem(const void* kern, size_t smem) {
+  static std::mutex mu;
+  std::lock_guard<std::mutex> lk(mu);
+  cudaFuncAttributes fa;
+  const bool ok =
+      cudaFuncGetAttributes(&fa, kern) == cudaSuccess &&
+      ((size_t)fa.maxDynamicSharedSizeBytes >= smem ||
+       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
+           cudaSuccess);
+  if (!ok) cudaGetLastError();
+  return ok;
+}
+
 static std::mutex g_pin_mu;
 static std::multimap<size_t, void*> g_pin_free;
 

@@ -197,6 +197,16 @@ void* host_pinned_get(size_t bytes);
 void host_pinned_put(void* p, size_t bytes);
 constexpr size_t PINNED_RED_BYTES = (size_t)RED_MAX_CTAS * 64 * sizeof(double);
 
+// Lets kern be launched with smem bytes of dynamic shared memory; false when the
+// device refuses. The limit belongs to the process and not to the call: it is only
+// ever raised, under a lock, so that no thread lowers what another one is about to
+// launch with.
+bool allow_smem(const void* kern, size_t smem);
+template <typename K>
+bool allow_smem(K kern, size_t smem) {
+  return allow_smem(reinterpret_cast<const void*>(kern), smem);
+}
+
 // error helpers -------------------------------------------------------------
 hs_status fail(hs_handle* hd, hs_status st, const std::string& msg);
 #define HS_CUDA_TRY(hd, call)                                                   \

@@ -231,10 +231,7 @@ static size_t smem_of(const hs_handle* hd) {
 
 template <typename K>
 static hs_status prep_smem(hs_handle* hd, K kern, size_t bytes) {
-  if (bytes > 48 * 1024)
-    HS_CUDA_TRY(hd, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)bytes));
-  return HS_OK;
+  return allow_smem(kern, bytes) ? HS_OK : fail(hd, HS_CUDA, "shared memory refused");
 }
 
 hs_status launch_matvec(hs_handle* hd, const void* x, void* y, hs_dtype dt, int shifted) {

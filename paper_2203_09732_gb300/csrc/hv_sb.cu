@@ -84,8 +84,7 @@ static hs_status make_dev(hs_handle* hd, int KS, DevPlan** out) {
   d->smem = smem_bytes<T>((int)P.low.size(), P.km);
   auto kern = kernel_of<T>(P.km);
   int nb = 0;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d->smem) ==
-          cudaSuccess &&
+  if (allow_smem(kern, d->smem) &&
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, NT_SB, d->smem) == cudaSuccess &&
       nb > 0) {
     d->grid = std::min(g.npairs, nb * hd->num_sms);
@@ -181,8 +180,7 @@ static hs_status make_dev4(hs_handle* hd, int KS, DevPlan4** out) {
   auto kern = kernel4_for<T, sb::MODE_HV>(g.km);
   const int nt = sizeof(T) == 8 ? NT4_D : NT4_F;
   int nb = 0;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d->smem) ==
-          cudaSuccess &&
+  if (allow_smem(kern, d->smem) &&
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, nt, d->smem) == cudaSuccess &&
       nb > 0) {
     d->grid = std::min(g.npairs, nb * hd->num_sms);
@@ -245,8 +243,7 @@ static hs_status make_dev6(hs_handle* hd, int KS, DevPlan6** out) {
   d->smem = smem_bytes6<T>(g.km);
   auto kern = kernel6<T, sb::MODE_HV>();
   int nb = 0;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d->smem) ==
-          cudaSuccess &&
+  if (allow_smem(kern, d->smem) &&
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, NT6, d->smem) == cudaSuccess &&
       nb > 0) {
     d->grid = std::min(g.npairs, nb * hd->num_sms);

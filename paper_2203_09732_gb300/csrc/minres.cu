@@ -395,15 +395,9 @@ static void enqueue_iters(hs_handle* hd, const MinresVecs& v, int iters, cudaStr
 template <typename T, int PC>
 static hs_status set_attrs(hs_handle* hd) {
   const size_t sm = row_smem_bytes<T>((int)hd->low.size());
-  if (sm > 48 * 1024) {
-    HS_CUDA_TRY(hd, cudaFuncSetAttribute(k_minres_init<T, PC>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    HS_CUDA_TRY(hd, cudaFuncSetAttribute(k_minres_A<T, PC>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    HS_CUDA_TRY(hd, cudaFuncSetAttribute(k_minres_B<T, PC>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  }
-  return HS_OK;
+  return allow_smem(k_minres_init<T, PC>, sm) && allow_smem(k_minres_A<T, PC>, sm) &&
+                 allow_smem(k_minres_B<T, PC>, sm)
+             ? HS_OK : fail(hd, HS_CUDA, "shared memory refused");
 }
 
 // Iterations per captured graph: more for small (latency-bound) problems.
@@ -487,11 +481,7 @@ static hs_status launch2_t(int device, cudaStream_t s, const SmemJob& job0,
   size_t sm = smr_bytes<T>(q[0].nlow, hc[0], q[0].rows_cap, NT);
   if (ng[1] > 0) sm = std::max(sm, smr_bytes<T>(q[1].nlow, hc[1], q[1].rows_cap, NT));
   if (sm + SMEM_STATIC_BYTES > (size_t)optin) return HS_CUDA;
-  if (cudaFuncSetAttribute(k_minres_smem<T, PC, JM, NT>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess) {
-    cudaGetLastError();
-    return HS_CUDA;
-  }
+  if (!allow_smem(k_minres_smem<T, PC, JM, NT>, sm)) return HS_CUDA;
   SmemJob j = job0;
   SmemQueue q0 = q[0], q1 = ng[1] > 0 ? q[1] : q[0];
   int ctas0 = ng[0] * q[0].S;
@@ -600,12 +590,7 @@ template <typename T, int PC>
 static hs_status solve_persist(hs_handle* hd, const T* b, const MinresVecs& v, double tol,
                                long long kmax) {
   const size_t sm = row_smem_bytes<T>((int)hd->low.size());
-  if (sm > 48 * 1024 &&
-      cudaFuncSetAttribute(k_minres_persist<T, PC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)sm) != cudaSuccess) {
-    cudaGetLastError();
-    return HS_CUDA;
-  }
+  if (!allow_smem(k_minres_persist<T, PC>, sm)) return HS_CUDA;
   const int grid = persist_grid<T, PC>(hd, sm);
   if (grid < 1) return HS_CUDA;
   Geo g = hd->geo();

@@ -396,11 +396,7 @@ hs_status launch1_t(int device, cudaStream_t s, const SmemJob& job0, const SmemQ
   size_t sm = smr1_bytes<T>(q[0].nlow, hc[0], q[0].rows_cap, NT);
   if (ng[1] > 0) sm = std::max(sm, smr1_bytes<T>(q[1].nlow, hc[1], q[1].rows_cap, NT));
   if (sm + SMEM_STATIC_BYTES > (size_t)optin) return HS_CUDA;
-  if (cudaFuncSetAttribute(k_minres_smem1<T, PC, JM, NT>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess) {
-    cudaGetLastError();
-    return HS_CUDA;
-  }
+  if (!allow_smem(k_minres_smem1<T, PC, JM, NT>, sm)) return HS_CUDA;
   SmemJob j = job0;
   SmemQueue q0 = q[0], q1 = ng[1] > 0 ? q[1] : q[0];
   int ctas0 = ng[0] * q[0].S;

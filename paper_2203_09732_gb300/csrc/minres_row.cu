@@ -347,8 +347,7 @@ hs_status row_launch(hs_handle* hd, const void* kern, int G, int nt, size_t smem
   int optin = 0;
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, hd->device);
   if (smem + fixed > (size_t)optin) return HS_CUDA;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-          cudaSuccess ||
+  if (!allow_smem(kern, smem) ||
       cudaLaunchCooperativeKernel(kern, dim3(G), dim3(nt), args, smem, hd->stream) != cudaSuccess) {
     cudaGetLastError();
     return HS_CUDA;

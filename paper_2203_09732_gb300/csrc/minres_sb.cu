@@ -59,8 +59,7 @@ auto kern_R() { return sb::k_sbrows<T, PC, MODE, NT_R>; }
 template <typename K>
 int grid_of(hs_handle* hd, K kern, int nt, size_t smem, int npairs) {
   int per_sm = 0;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-          cudaSuccess ||
+  if (!allow_smem(kern, smem) ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem) != cudaSuccess) {
     cudaGetLastError();
     return 0;

@@ -848,11 +848,7 @@ hs_status launch_sweep_t(int device, cudaStream_t s, const SweepArgs (&a)[2],
   if (ng[1] > 0) sm = std::max(sm, smr_bytes<double>(q[1].nlow, hc[1], q[1].rows_cap, NT));
   sm += SWEEP_SCRATCH;
   if (sm + fa.sharedSizeBytes > (size_t)optin) return HS_CUDA;
-  if (cudaFuncSetAttribute(k_sweep<PC, JM, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)sm) != cudaSuccess) {
-    cudaGetLastError();
-    return HS_CUDA;
-  }
+  if (!allow_smem(k_sweep<PC, JM, NT>, sm)) return HS_CUDA;
   SweepArgs a0 = a[0], a1 = ng[1] > 0 ? a[1] : a[0];
   SmemQueue q0 = q[0], q1 = ng[1] > 0 ? q[1] : q[0];
   int ctas0 = ng[0] * q[0].S;

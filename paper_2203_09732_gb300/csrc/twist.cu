@@ -93,9 +93,7 @@ hs_status launch_twist(hs_handle* hd, const double* psi, int K, double* z_host) 
   if (st != HS_OK) return st;
   const int L = hd->L;
   const size_t sm = tw_smem(L);
-  if (sm + TW_LOW > 48 * 1024)   // with the static table
-    HS_CUDA_TRY(hd, cudaFuncSetAttribute(k_twist, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sm));
+  if (!allow_smem(k_twist, sm)) return fail(hd, HS_CUDA, "hs_twist: shared memory");
   // CTAs per vector: about three per SM in all, at least four blocks a warp; the
   // sums of a launch's vectors first in the scratch, then the CTAs' bins
   constexpr int KB = 64;
