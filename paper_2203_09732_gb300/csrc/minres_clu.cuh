@@ -669,7 +669,7 @@ inline bool clu_launch(K kern, int grid, int cs, size_t smem, cudaStream_t s, A.
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  if (!allow_smem(kern, smem) ||
+  if (cs < 1 || cs > CLU_SIZE_MAX || !allow_smem(kern, smem) ||
       (cs > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
                      cudaSuccess) ||
       cudaLaunchKernelEx(&cfg, kern, args...) != cudaSuccess) {

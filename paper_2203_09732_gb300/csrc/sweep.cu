@@ -773,8 +773,9 @@ double clu_iter_us(long long n, int cs) { return 1.5 + 0.8 * clu_rpt((int)n, cs)
 
 // The cluster size for a sweep, at least smin: the one whose clusters finish a
 // list of realisations (longest first, each to the cluster that is free first)
-// soonest by clu_iter_us. Work per realisation: about n^1.05 iterations a solve.
+// soonest by clu_iter_us (HS_MINRES_CLUSTER forces it). Work per realisation: about n^1.05 iterations a solve.
 int clu_sweep_size(const std::vector<long long>& ns, int num_sms, int smin) {
+  if (const char* e = getenv("HS_MINRES_CLUSTER")) return clu_rpt((int)ns[0], atoi(e)) ? atoi(e) : 0;
   int best = 0;
   double best_t = 1e300;
   for (int cs = 1; cs <= CLU_SIZE_MAX && cs <= num_sms; cs *= 2) {
@@ -989,49 +990,117 @@ extern "C" hs_status hs_sweep(int B, const int* L_host, const double* h_host, in
   }
   if (cudaMalloc(&err, sizeof(int)) != cudaSuccess) return cleanup(HS_OOM);
   if (cudaMemsetAsync(err, 0, sizeof(int), s) != cudaSuccess) return cleanup(HS_CUDA);
-  // short chains: one cluster per realisation at a time
-  bool clu = !getenv("HS_SWEEP_S");
-  for (int r = 0; r < B; ++r)
-    clu = clu && hd[r]->n <= CLU_F64_ROWS && clu_choice(hd[r]->n, num_sms) > 0;
-  // group size per class: forced (HS_SWEEP_S), cached or timed
+  // one kernel shape per launch: the rows-per-lane template follows k <= 8
+  for (int c = 0; c < ncls; ++c) {
+    cls[c].hd0 = hd[cls[c].idx[0]];
+    cls[c].n = cls[c].hd0->n;
+  }
+  const int k_lo = cls[0].hd0->k;
+  for (int c = 1; c < ncls; ++c)
+    if ((cls[c].hd0->k <= 8) != (k_lo <= 8)) return cleanup(HS_BAD_ARG);
+  // group size of a class: forced (HS_SWEEP_S), cached or timed; HS_CUDA when none runs
   auto tunes = tune_read();
   bool tunes_changed = false;
-  for (int c = 0; c < ncls; ++c) {
-    Class& C = cls[c];
-    C.hd0 = hd[C.idx[0]];
-    C.n = C.hd0->n;
-    if (!clu && (st = alloc_class(C, num_sms)) != HS_OK) return cleanup(st);
+  auto tune = [&](Class& C, bool clusters) -> hs_status {
+    C.tune = Tune();
     char key[96];
-    snprintf(key, sizeof key, "L%d_pc%d_f64_%ssm%d", C.L, (int)pc, clu ? "clu_" : "", num_sms);
+    snprintf(key, sizeof key, "L%d_pc%d_f64_%ssm%d", C.L, (int)pc, clusters ? "clu_" : "", num_sms);
+    const int most = clusters ? CLU_SIZE_MAX : num_sms;
     if (const char* fs = getenv("HS_SWEEP_S")) {
       C.tune.S = std::max(1, std::min(num_sms, atoi(fs)));
       C.tune.rate = 1.0;
       C.tuned = -1;
-    } else if (tunes.count(key)) {
+    } else if (tunes.count(key) && tunes[key].S >= 1 && tunes[key].S <= most) {
       C.tune = tunes[key];
       C.tuned = 0;
     } else {
-      st = clu ? tune_clu(runs[C.idx[0]], pc, num_sms, s, &C.tune)
-               : tune_class(C, runs, pc, num_sms, device, s, err, 0);
-      if (st == HS_OK && !C.tune.S) st = HS_CUDA;
-      if (st != HS_OK) return cleanup(st);
+      hs_status t = clusters ? tune_clu(runs[C.idx[0]], pc, num_sms, s, &C.tune)
+                             : tune_class(C, runs, pc, num_sms, device, s, err, 0);
+      if (t == HS_OK && !C.tune.S) t = HS_CUDA;
+      if (t != HS_OK) return t;
       C.tuned = 1;
       tunes[key] = C.tune;
       tunes_changed = true;
     }
     C.tune.one = 0;
+    return HS_OK;
+  };
+  double t_setup = 0.0;
+  auto ts = clk::now();
+  auto setup_done = [&] {
+    if (tunes_changed) tune_write(tunes);
+    tunes_changed = false;
+    ts = clk::now();
+    t_setup = std::chrono::duration<double>(ts - t0).count();
+  };
+  const unsigned long long limit = 1ull << 22;
+  // short chains: one cluster per realisation at a time, from one list of all of
+  // them, the longest chains first. Where no cluster runs or the launch is refused,
+  // the groups of CTAs below.
+  std::vector<int> list(B);
+  const size_t ab_bytes = sizeof(double) * 2 * SWEEP_MMAX * B, it_bytes = sizeof(long long) * B,
+               res_bytes = sizeof(int) * 4 * B, re_bytes = (sizeof(SweepReal) * B + 15) & ~size_t(15);
+  auto run_clusters = [&]() -> hs_status {
+    int smin = 1;
+    for (int c = 0; c < ncls; ++c) {
+      const hs_status t = tune(cls[c], true);
+      if (t != HS_OK) return t;
+      smin = std::max(smin, cls[c].tune.S);
+    }
+    for (int r = 0; r < B; ++r) list[r] = r;
+    std::stable_sort(list.begin(), list.end(), [&](int a, int b) { return hd[a]->n > hd[b]->n; });
+    std::vector<long long> ns(B);
+    for (int j = 0; j < B; ++j) ns[j] = hd[list[j]]->n;
+    const int cs = clu_sweep_size(ns, num_sms, std::min(smin, num_sms));
+    if (cs < 1) return HS_CUDA;
+    const int groups = std::min(B, std::max(1, num_sms / cs));
+    size_t sm = 0;
+    for (int c = 0; c < ncls; ++c) {
+      sm = std::max(sm, clu_bytes<double>((int)cls[c].n, cls[c].L, cs, clu_rpt((int)cls[c].n, cs)));
+      cls[c].tune.S = cs;
+      cls[c].ngroups = groups;
+    }
+    hs_status t = dev_alloc(hd[0], (void**)&cmem, ab_bytes + it_bytes + res_bytes + re_bytes + 16);
+    if (t != HS_OK) return t;
+    double* ab = reinterpret_cast<double*>(cmem);
+    long long* its = reinterpret_cast<long long*>(cmem + ab_bytes);
+    int* res = reinterpret_cast<int*>(cmem + ab_bytes + it_bytes);
+    int* head = reinterpret_cast<int*>(cmem + ab_bytes + it_bytes + res_bytes);
+    char* reals = cmem + ab_bytes + it_bytes + res_bytes + 16;
+    std::vector<SweepReal> hr(B);
+    for (int j = 0; j < B; ++j) {
+      const int r = list[j];
+      hr[j] = SweepReal{hd[r]->geo(), hd[r]->sigma, runs[r].V, runs[r].x, runs[r].w,
+                        ab + (size_t)2 * SWEEP_MMAX * j, ab + (size_t)2 * SWEEP_MMAX * j + SWEEP_MMAX,
+                        nullptr, res + 4 * j, its + j, runs[r].m};
+    }
+    // pageable source: staged before the call returns
+    if (cudaMemsetAsync(cmem + ab_bytes, 0, it_bytes + res_bytes + 16, s) != cudaSuccess ||
+        cudaMemcpyAsync(reals, hr.data(), sizeof(SweepReal) * B, cudaMemcpyHostToDevice, s) !=
+            cudaSuccess) {
+      cudaGetLastError();
+      return fail(hd[0], HS_CUDA, "hs_sweep: upload failed");
+    }
+    setup_done();
+    return clu_launch(k_sweep_clu, groups * cs, cs, sm, s, reinterpret_cast<const SweepReal*>(reals), B,
+                      head, K, tol, minres_tol, (int)pc, clu_limit())
+               ? HS_OK : HS_CUDA;
+  };
+  bool clu = !getenv("HS_SWEEP_S");
+  for (int r = 0; r < B; ++r)
+    clu = clu && hd[r]->n <= CLU_F64_ROWS && clu_choice(hd[r]->n, num_sms) > 0;
+  hs_status ls = HS_CUDA;
+  if (clu) {
+    ls = run_clusters();
+    if (ls != HS_OK && ls != HS_CUDA) return cleanup(ls);
+    clu = ls == HS_OK;
   }
-  if (tunes_changed) tune_write(tunes);
-  // one kernel shape per launch: the rows-per-lane template follows k <= 8
-  const int k_lo = cls[0].hd0->k;
-  for (int c = 1; c < ncls; ++c)
-    if ((cls[c].hd0->k <= 8) != (k_lo <= 8)) return cleanup(HS_BAD_ARG);
-  // realisation records
-  for (int c = 0; c < ncls; ++c) {
+  // the groups of CTAs: their sizes, buffers and realisation records
+  for (int c = 0; c < ncls && !clu; ++c) {
     Class& C = cls[c];
+    if ((st = alloc_class(C, num_sms)) != HS_OK || (st = tune(C, false)) != HS_OK) return cleanup(st);
     Dev& D = dv[c];
     const int nr = (int)C.idx.size();
-    if (clu) continue;
     if (cudaMalloc(&D.reals, sizeof(SweepReal) * nr) != cudaSuccess ||
         cudaMalloc(&D.ab, sizeof(double) * 2 * SWEEP_MMAX * nr) != cudaSuccess ||
         cudaMalloc(&D.res, sizeof(int) * 4 * nr) != cudaSuccess ||
@@ -1069,60 +1138,9 @@ extern "C" hs_status hs_sweep(int B, const int* L_host, const double* h_host, in
       return cleanup(HS_CUDA);
     }
   }
-  // the cluster form: one list of all realisations, the longest chains first
-  std::vector<int> list(B);
-  const size_t ab_bytes = sizeof(double) * 2 * SWEEP_MMAX * B, it_bytes = sizeof(long long) * B,
-               res_bytes = sizeof(int) * 4 * B, re_bytes = (sizeof(SweepReal) * B + 15) & ~size_t(15);
-  int* chead = nullptr;
-  if (clu) {
-    for (int r = 0; r < B; ++r) list[r] = r;
-    std::stable_sort(list.begin(), list.end(), [&](int a, int b) { return hd[a]->n > hd[b]->n; });
-    if ((st = dev_alloc(hd[0], (void**)&cmem, ab_bytes + it_bytes + res_bytes + re_bytes + 16)) !=
-        HS_OK)
-      return cleanup(st);
-    double* ab = reinterpret_cast<double*>(cmem);
-    long long* its = reinterpret_cast<long long*>(cmem + ab_bytes);
-    int* res = reinterpret_cast<int*>(cmem + ab_bytes + it_bytes);
-    chead = reinterpret_cast<int*>(cmem + ab_bytes + it_bytes + res_bytes);
-    std::vector<SweepReal> hr(B);
-    for (int j = 0; j < B; ++j) {
-      const int r = list[j];
-      hr[j] = SweepReal{hd[r]->geo(), hd[r]->sigma, runs[r].V, runs[r].x, runs[r].w,
-                        ab + (size_t)2 * SWEEP_MMAX * j, ab + (size_t)2 * SWEEP_MMAX * j + SWEEP_MMAX,
-                        nullptr, res + 4 * j, its + j, runs[r].m};
-    }
-    if (cudaMemsetAsync(cmem + ab_bytes, 0, it_bytes + res_bytes + 16, s) != cudaSuccess ||
-        cudaMemcpyAsync(cmem + ab_bytes + it_bytes + res_bytes + 16, hr.data(),
-                        sizeof(SweepReal) * B, cudaMemcpyHostToDevice, s) != cudaSuccess) {
-      cudaGetLastError();
-      return cleanup(HS_CUDA);
-    }
-  }
-  const double t_setup = std::chrono::duration<double>(clk::now() - t0).count();
   // the launch: groups per class from the split of the SMs; a group size that
   // does not fit the kernel's shared memory grows by one CTA until it fits
-  const auto ts = clk::now();
-  const unsigned long long limit = 1ull << 22;
-  hs_status ls = HS_CUDA;
-  if (clu) {
-    std::vector<long long> ns(B);
-    for (int j = 0; j < B; ++j) ns[j] = hd[list[j]]->n;
-    int smin = 1;
-    for (int c = 0; c < ncls; ++c) smin = std::max(smin, cls[c].tune.S);
-    const int cs = clu_sweep_size(ns, num_sms, std::min(smin, num_sms));
-    const int groups = cs > 0 ? std::min(B, num_sms / cs) : 0;
-    size_t sm = 0;
-    for (int c = 0; c < ncls && cs > 0; ++c) {
-      sm = std::max(sm, clu_bytes<double>((int)cls[c].n, cls[c].L, cs, clu_rpt((int)cls[c].n, cs)));
-      cls[c].tune.S = cs;
-      cls[c].ngroups = groups;
-    }
-    if (cs > 0 &&
-        clu_launch(k_sweep_clu, groups * cs, cs, sm, s,
-                   reinterpret_cast<const SweepReal*>(cmem + ab_bytes + it_bytes + res_bytes + 16), B,
-                   chead, K, tol, minres_tol, (int)pc, clu_limit()))
-      ls = HS_OK;
-  }
+  if (!clu) setup_done();
   for (int attempt = 0; !clu && attempt < 64 && ls == HS_CUDA; ++attempt) {
     split_groups(cls, ncls, num_sms);
     int used = 0;
