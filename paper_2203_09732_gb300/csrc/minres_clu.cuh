@@ -55,6 +55,7 @@ struct CluShared {
   struct { double co[4]; int apply, stop; } d[2];   // D: cq, cd1, cd2, tau (of type T)
   int fail;                                     // a wait of this CTA gave up
   int gave_up;                                  // a wait of any CTA did (clu_agree)
+  unsigned phase[4];                            // compute warps' parities after a solve: b, c, d
   MinresState S;                                // the solve's state (rotation warp)
 };
 
@@ -142,7 +143,9 @@ __host__ __device__ inline size_t clu_bytes(int n, int L, int cs, int rpt) {
 }
 
 // Phase parities of a cluster's barriers, carried from solve to solve, and the
-// polls of a wait.
+// polls of a wait. Every warp keeps its own; a compute warp without rows in a
+// solve waits for nothing in it and takes compute warp 0's at its end, so solves
+// of one kernel may follow each other in any order of sizes.
 struct CluPhase {
   unsigned limit;
   unsigned a = 0, b = 0, c = 0, d[2] = {0, 0}, e[2] = {0, 0}, f[2] = {0, 0};
@@ -525,6 +528,10 @@ __device__ bool clu_solve(const SmemJob& job, int pc, CluShared& sh, char* dyn, 
 #pragma unroll
     for (int j = 0; j < RPT; ++j)
       if (xo && owned(j)) xo[r0 + lrow(j)] = x[j];
+    if (t0 == 0) {
+      sh.phase[0] = ph.b; sh.phase[1] = ph.c;
+      sh.phase[2] = ph.d[0]; sh.phase[3] = ph.d[1];
+    }
   } else if (wid == -1) {
     // ---- beta warp
     double ib = 1.0;                             // 1 / beta_{k-1} (beta_0 = 1)
@@ -627,6 +634,10 @@ __device__ bool clu_solve(const SmemJob& job, int pc, CluShared& sh, char* dyn, 
     if (lane == 0) sh.S = S;
   }
   __syncthreads();
+  if (wid >= nwa) {
+    ph.b = sh.phase[0]; ph.c = sh.phase[1];
+    ph.d[0] = sh.phase[2]; ph.d[1] = sh.phase[3];
+  }
   const bool ok = clu_agree(sh);
   if (threadIdx.x == 0) {
     if (!ok) sh.S.status = HS_TIMEOUT;
