@@ -92,16 +92,19 @@ __device__ __forceinline__ void bar_arrive(unsigned long long* b) {
   asm volatile("mbarrier.arrive.shared.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
 }
 // Waits for the phase of the given parity (whole warps); false in every lane
-// once any lane has polled limit times in vain.
+// after limit polls. The vote that makes the answer the warp's is the loop's only
+// branch: with a vote behind a loop per lane an iteration took 4 to 9 % longer.
 __device__ __forceinline__ bool bar_wait(unsigned long long* b, unsigned parity, unsigned limit) {
   const uint32_t a = smem_u32(b);
-  uint32_t done = 0;
-  for (unsigned it = 0; it < limit && !done; ++it)
+  for (unsigned it = 0; it != limit; ++it) {
+    uint32_t done;
     asm volatile("{\n.reg .pred p;\n"
                  "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
                  "selp.u32 %0, 1, 0, p;\n}"
                  : "=r"(done) : "r"(a), "r"(parity) : "memory");
-  return __all_sync(0xffffffffu, done);
+    if (__all_sync(0xffffffffu, done)) return true;
+  }
+  return false;
 }
 // One or two values into another CTA's shared memory, counted by its mbarrier.
 __device__ __forceinline__ void clu_send(uint32_t dst, double v, uint32_t bar) {
@@ -199,15 +202,18 @@ __device__ __forceinline__ double clu_total(const double* slot, int np) {
 static_assert(CLU_SIZE_MAX * CLU_NW <= 64, "clu_total adds two partials per lane");
 
 // alpha_k = q_k . p_k / beta_k^2 in odd lanes, alpha_k / beta_k in even ones, from
-// q_k . p_k (doubled) and the words of F. 1 / (2 beta_k^3) leaves the range of
-// doubles where beta_k is beyond 1e102 or below 1e-103 (a right-hand side that
-// large or small; H that large): from 2^+-330 on the quotient takes two steps.
-__device__ __forceinline__ double clu_alpha(const double* f, double qp2) {
+// q_k . p_k (doubled) and the words of F. beta_1 carries the scale of the right-hand
+// side, and 1 / (2 beta_1^3) leaves the range of doubles beyond 1e102 and below
+// 1e-103: from 2^+-330 on the quotient takes two steps there. (The later beta_k are
+// on the scale of M^-1 H, whose q . p overflows first.)
+__device__ __forceinline__ double clu_alpha(const double* f, int k, double qp2) {
   const bool odd = threadIdx.x & 1;
-  const double ib = f[3];
-  const bool wide = ((unsigned)__double2hiint(ib) >> 20) - (1023u - 330u) > 660u;
-  const double a = qp2 * f[odd || wide ? 4 : 5];
-  return wide && !odd ? a * ib : a;
+  if (k == 1) {
+    const double ib = f[3];
+    if (((unsigned)__double2hiint(ib) >> 20) - (1023u - 330u) > 660u)
+      return odd ? qp2 * f[4] : qp2 * f[4] * ib;
+  }
+  return qp2 * f[odd ? 4 : 5];
 }
 
 // The Givens rotation of step k (Algorithm 2) and its d/x coefficients: the
@@ -589,7 +595,7 @@ __device__ bool clu_solve(const SmemJob& job, int pc, CluShared& sh, char* dyn, 
         }
         continue;
       }
-      const double al = clu_alpha(sh.f[t], tot);
+      const double al = clu_alpha(sh.f[t], k, tot);
       if (lane == 0) {
         T* co = reinterpret_cast<T*>(sh.c);
         co[0] = (T)sh.f[t][3]; co[1] = (T)al; co[2] = (T)sh.f[t][6];

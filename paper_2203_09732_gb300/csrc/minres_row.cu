@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(ROW_NT, 1) k_minres_row(RowArgs ra, int pc) {
         if (sh.d[0].stop) break;
         continue;
       }
-      const double al = clu_alpha(sh.f[t], tot);
+      const double al = clu_alpha(sh.f[t], k, tot);
       if (lane == 0) {
         T* co = reinterpret_cast<T*>(sh.c);
         co[0] = (T)sh.f[t][3]; co[1] = (T)al; co[2] = (T)sh.f[t][6];

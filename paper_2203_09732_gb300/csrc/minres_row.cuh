@@ -22,15 +22,16 @@ struct RowArgs {
 // set fail.
 __device__ __forceinline__ bool row_wait(int& fail, unsigned long long* b, unsigned parity) {
   const uint32_t a = smem_u32(b);
-  uint32_t done = 0;
-  for (unsigned it = 0; it < CLU_WAIT_LIMIT && !done; ++it) {
+  for (unsigned it = 0; it != CLU_WAIT_LIMIT; ++it) {
+    uint32_t done;
     asm volatile("{\n.reg .pred p;\n"
                  "mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2;\n"
                  "selp.u32 %0, 1, 0, p;\n}"
                  : "=r"(done) : "r"(a), "r"(parity) : "memory");
-    if ((it & 15u) == 15u && !done && *(volatile int*)&fail) break;
+    if (__all_sync(0xffffffffu, done)) return true;
+    if ((it & 15u) == 15u && __any_sync(0xffffffffu, *(volatile int*)&fail)) return false;
   }
-  return __all_sync(0xffffffffu, done);
+  return false;
 }
 
 // A wait of this warp gave up: the CTA's other warps stop waiting, and the host
