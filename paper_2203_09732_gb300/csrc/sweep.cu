@@ -651,7 +651,7 @@ __global__ void __launch_bounds__(CLU_NT, 1) k_sweep_clu(const SweepReal* reals,
     int k = 0, unconv = 0, status = HS_OK;
     long long iters = 0;
     double bk = 0.0;
-    bool done = false, skip = false;
+    bool done = false;
     while (!done) {
       const double* vk = sr.V + (size_t)k * n;
       // (H - sigma) x = v_k
@@ -720,20 +720,13 @@ __global__ void __launch_bounds__(CLU_NT, 1) k_sweep_clu(const SweepReal* reals,
       double pb = 0.0;
       for (long long i = lo + threadIdx.x; i < hi; i += NT) pb += sr.w[i] * sr.w[i];
       const double bn = sqrt(fmax(clu_sum(sh, pb, turn), 0.0));
-      // the convergence test (every CTA's thread 0 on the same numbers). It takes
-      // about as long as 0.3 kk^2 iterations of a solve, so the step after one that
-      // left two pairs or more open goes without
+      // the convergence test (every CTA's thread 0 on the same numbers)
       if (threadIdx.x == 0) {
         sh.alpha[k] = al;
         const int kk = k + 1;
         const bool last = bn <= 1e-13 * fabs(al) || kk == sr.m;
         int nconv = 0;
-        if (kk >= K && (last || !skip)) {
-          nconv = ritz_converged(kk, sh.alpha, sh.beta, bn, K, tol, sh.qd, sh.qe, sh.qz);
-          skip = nconv < K - 1;
-        } else {
-          skip = false;
-        }
+        if (kk >= K) nconv = ritz_converged(kk, sh.alpha, sh.beta, bn, K, tol, sh.qd, sh.qe, sh.qz);
         const bool stop = nconv == K || last;
         sh.flag[0] = stop ? 1 : 0;
         sh.flag[1] = nconv;

@@ -62,3 +62,18 @@ def test_longest_with_short_chains(cs, tune_file, monkeypatch):
         monkeypatch.setenv("HS_MINRES_CLUSTER", cs)
     info = _sweep(hs, [14, 8, 14] + [8] * 40, 3)
     assert cs is None or info["S"] == [int(cs)] * 2
+
+
+def test_stops_at_the_same_step_as_the_groups(tune_file, monkeypatch):
+    """The convergence test on T_k follows every step in both forms: one realisation
+    at a time, ten pairs to a loose tolerance (two or more of them often converge in
+    one step), the same number of Lanczos steps."""
+    hs = need_gpu()
+    for r in range(6):
+        h = inputs.disorder(10, 3.0, 90 + r)
+        with monkeypatch.context() as m:
+            m.setenv("HS_SWEEP_S", "8")
+            groups = hs.sweep([10], [h], 10, tol=1e-2)[-1]
+        clusters = hs.sweep([10], [h], 10, tol=1e-2)[-1]
+        assert clusters["max_steps"] == groups["max_steps"]
+        assert clusters["converged"] == groups["converged"] == 1
