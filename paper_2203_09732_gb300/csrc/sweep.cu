@@ -23,6 +23,7 @@
 
 #include "lanczos.cuh"
 #include "minres_clu.cuh"
+#include "ql.cuh"
 
 namespace hs {
 
@@ -390,11 +391,8 @@ __device__ int ritz_converged(int kk, const double* alpha, const double* beta, d
       for (int i = m - 1; i >= l; --i) {
         const double f = s * e[i];
         const double b = cc * e[i];
-        // one reciprocal root for r, f / r and g / r (7 FP64 instructions; a
-        // hypot and two divisions are about 35, at 64 cycles each)
-        const double rr = f * f + g * g;
-        const double ir = rr > 0.0 ? rsqrt(rr) : 0.0;
-        r = rr * ir;
+        double sn, cs;
+        ql_rotation(f, g, r, sn, cs);
         e[i + 1] = r;
         if (r == 0.0) {
           d[i + 1] -= p;
@@ -402,8 +400,8 @@ __device__ int ritz_converged(int kk, const double* alpha, const double* beta, d
           underflow = true;
           break;
         }
-        s = f * ir;
-        cc = g * ir;
+        s = sn;
+        cc = cs;
         g = d[i + 1] - p;
         r = (d[i] - g) * s + 2.0 * cc * b;
         p = s * r;
