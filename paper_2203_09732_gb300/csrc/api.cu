@@ -48,8 +48,21 @@ hs_status dev_alloc(hs_handle* hd, void** p, size_t bytes) {
   *p = nullptr;
   if (bytes == 0) bytes = 256;
   cudaMemPool_t pool = pool_for(hd->device);
-  const cudaError_t e = pool ? cudaMallocFromPoolAsync(p, bytes, pool, hd->stream)
-                             : cudaMalloc(p, bytes);
+  auto get = [&] {
+    return pool ? cudaMallocFromPoolAsync(p, bytes, pool, hd->stream) : cudaMalloc(p, bytes);
+  };
+  cudaError_t e = get();
+  if (e != cudaSuccess && hd->sb_m) {
+    // what the handle keeps for speed goes first (minres_sb.cu: M and 1/M, which the
+    // captured chunks point to; the next solve makes both again where there is room)
+    cudaGetLastError();
+    sb_graphs_release(hd, 1);
+    dev_free(hd, hd->sb_m);
+    hd->sb_m = nullptr;
+    cudaStreamSynchronize(hd->stream);
+    if (pool) cudaMemPoolTrimTo(pool, 0);
+    e = get();
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     *p = nullptr;
