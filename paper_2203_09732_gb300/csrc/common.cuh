@@ -160,10 +160,14 @@ struct hs_handle {
   int smr_grid = 0, smr_rows_cap = 0, smr_hdr_cap = 0;
   int* d_smr_first = nullptr;
 
-  // superblock H x plans (hv_sb.cu): [0] FP32, [1] FP64; null where not built
+  // superblock plans (hv_sb.cu): [0] FP32, [1] FP64; null where not built. Ten low
+  // bits (sb.cuh) and four (sb4.cuh): sb_ten and sb_four make those that the defaults
+  // seldom or never use at their first use, with the windows (-1: no plan, or it
+  // was tried) of the handle's creation.
   void* sb_plan[2] = {nullptr, nullptr};
-  // four-low-bit superblock plans (sb4.cuh): [0] FP32, [1] FP64
   void* sb4_plan[2] = {nullptr, nullptr};
+  int sb_ks[2] = {-1, -1}, sb4_ks[2] = {-1, -1};
+  bool sb_on = false;                // the chain takes superblock plans
   // six-low-bit superblock plan (sb6.cuh, FP64)
   void* sb6_plan = nullptr;
   // superblock MINRES chunk graphs (minres_sb.cu), [precision][preconditioner],
@@ -222,6 +226,10 @@ hs_status launch_matvec(hs_handle* hd, const void* x, void* y, hs_dtype dt, int 
 // hv_sb.cu: superblock form for long chains; *used = false if it does not apply
 hs_status sb_setup(hs_handle* hd);
 void sb_release(hs_handle* hd);
+// the ten- and four-low-bit plans (sb::DevPlan, sb4::DevPlan4) of precision ti (0
+// FP32, 1 FP64), made now if need be; null where none applies
+void* sb_ten(hs_handle* hd, int ti);
+void* sb_four(hs_handle* hd, int ti);
 hs_status launch_matvec_sb(hs_handle* hd, const void* x, void* y, hs_dtype dt, int shifted,
                            bool* used);
 hs_status launch_unrank(hs_handle* hd, long long first, long long count, unsigned int* out);

@@ -261,28 +261,28 @@ static hs_status make_dev6(hs_handle* hd, int KS, DevPlan6** out) {
 // slots and sums of a pair take 65 KB in FP32, two CTAs per SM) and at most
 // L - 10 bits, so that a chain has at least 512 superblock pairs to spread
 // over the GPU. HS_SB_KS32 and HS_SB_KS64 override the window (tuning).
+// The defaults need the FP64 plans of ten bits (initial pass) and of six (pass A)
+// only; the others are made here if the environment asks for their forms now (a
+// capture then finds them), else at their first use (hs_create at L = 24 and 28: 5.8
+// and 73.2 ms with all made here, 3.7 and 65.2 so).
 hs_status sb_setup(hs_handle* hd) {
-  int ks32 = std::min(hd->k + 4, hd->L - 10), ks64 = std::min(hd->k + 3, hd->L - 10);
-  if (const char* e = getenv("HS_SB_KS32")) ks32 = atoi(e);
-  if (const char* e = getenv("HS_SB_KS64")) ks64 = atoi(e);
-  sb::DevPlan* d = nullptr;
-  hs_status st = sb::make_dev<float>(hd, ks32, &d);
-  if (st != HS_OK) return st;
-  hd->sb_plan[0] = d;
-  st = sb::make_dev<double>(hd, ks64, &d);
-  if (st != HS_OK) return st;
-  hd->sb_plan[1] = d;
+  hd->sb_on = true;
+  hd->sb_ks[0] = std::min(hd->k + 4, hd->L - 10);
+  hd->sb_ks[1] = std::min(hd->k + 3, hd->L - 10);
+  if (const char* e = getenv("HS_SB_KS32")) hd->sb_ks[0] = atoi(e);
+  if (const char* e = getenv("HS_SB_KS64")) hd->sb_ks[1] = atoi(e);
   // four-low-bit plans (sb4.cuh): 14-bit windows in FP32, 13 in FP64 (the
   // slots and sums of a pair take about 96 KB either way); HS_SB4_KS32 and
   // HS_SB4_KS64 override them (tests of small chains)
-  int k32 = std::min(14, hd->L - 6), k64 = std::min(13, hd->L - 6);
-  if (const char* e = getenv("HS_SB4_KS32")) k32 = atoi(e);
-  if (const char* e = getenv("HS_SB4_KS64")) k64 = atoi(e);
-  sb4::DevPlan4* d4 = nullptr;
-  if ((st = sb4::make_dev4<float>(hd, k32, &d4)) != HS_OK) return st;
-  hd->sb4_plan[0] = d4;
-  if ((st = sb4::make_dev4<double>(hd, k64, &d4)) != HS_OK) return st;
-  hd->sb4_plan[1] = d4;
+  hd->sb4_ks[0] = std::min(14, hd->L - 6);
+  hd->sb4_ks[1] = std::min(13, hd->L - 6);
+  if (const char* e = getenv("HS_SB4_KS32")) hd->sb4_ks[0] = atoi(e);
+  if (const char* e = getenv("HS_SB4_KS64")) hd->sb4_ks[1] = atoi(e);
+  sb::DevPlan* d = nullptr;
+  hs_status st = sb::make_dev<double>(hd, hd->sb_ks[1], &d);
+  hd->sb_ks[1] = -1;
+  if (st != HS_OK) return st;
+  hd->sb_plan[1] = d;
   // six-low-bit plan (sb6.cuh, FP64): 13-bit windows (the slots and sums of a
   // pair take 97 KB; 12 and 11 bits leave more whole-superblock bonds to global
   // memory, L = 28: 2084 -> 2811 -> 3682 us); HS_SB6_KS overrides it (tests of
@@ -292,7 +292,42 @@ hs_status sb_setup(hs_handle* hd) {
   sb6::DevPlan6* d6 = nullptr;
   if ((st = sb6::make_dev6<double>(hd, j64, &d6)) != HS_OK) return st;
   hd->sb6_plan = d6;
+  if (getenv("HS_HV_SB") || getenv("HS_SB4")) sb_ten(hd, 0);
+  if (getenv("HS_SB4")) {
+    sb_four(hd, 0);
+    sb_four(hd, 1);
+  }
   return HS_OK;
+}
+
+// Whether plans can be made now (not while the stream is being captured).
+static bool can_make(hs_handle* hd) {
+  cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(hd->stream, &c) == cudaSuccess && c == cudaStreamCaptureStatusNone;
+}
+
+void* sb_ten(hs_handle* hd, int ti) {
+  if (!hd->sb_plan[ti] && hd->sb_ks[ti] >= 0 && can_make(hd)) {
+    sb::DevPlan* d = nullptr;
+    const hs_status st = ti ? sb::make_dev<double>(hd, hd->sb_ks[ti], &d)
+                            : sb::make_dev<float>(hd, hd->sb_ks[ti], &d);
+    if (st != HS_OK) hd->err.clear();   // no room: another form
+    hd->sb_ks[ti] = -1;
+    hd->sb_plan[ti] = d;
+  }
+  return hd->sb_plan[ti];
+}
+
+void* sb_four(hs_handle* hd, int ti) {
+  if (!hd->sb4_plan[ti] && hd->sb4_ks[ti] >= 0 && can_make(hd)) {
+    sb4::DevPlan4* d = nullptr;
+    const hs_status st = ti ? sb4::make_dev4<double>(hd, hd->sb4_ks[ti], &d)
+                            : sb4::make_dev4<float>(hd, hd->sb4_ks[ti], &d);
+    if (st != HS_OK) hd->err.clear();
+    hd->sb4_ks[ti] = -1;
+    hd->sb4_plan[ti] = d;
+  }
+  return hd->sb4_plan[ti];
 }
 
 void sb_release(hs_handle* hd) {
@@ -352,9 +387,9 @@ hs_status launch_matvec_sb(hs_handle* hd, const void* x, void* y, hs_dtype dt, i
     }
   }
   {
-    auto* d4 = static_cast<sb4::DevPlan4*>(hd->sb4_plan[dt == HS_F32 ? 0 : 1]);
+    auto* d4 = static_cast<sb4::DevPlan4*>(want == 4 ? sb_four(hd, dt == HS_F32 ? 0 : 1) : nullptr);
     const size_t es = dt == HS_F32 ? sizeof(float) : sizeof(double);
-    if (want == 4 && d4 && d4->ok && ((uintptr_t)x % es) == 0 && ((uintptr_t)y % es) == 0) {
+    if (d4 && d4->ok && ((uintptr_t)x % es) == 0 && ((uintptr_t)y % es) == 0) {
       const sb::MinresArgs none{};
       if (dt == HS_F32)
         sb4::kernel4_for<float, sb::MODE_HV>(d4->geo.km)<<<d4->grid, sb4::NT4_F, d4->smem,
@@ -372,7 +407,7 @@ hs_status launch_matvec_sb(hs_handle* hd, const void* x, void* y, hs_dtype dt, i
       return HS_OK;
     }
   }
-  auto* d = static_cast<sb::DevPlan*>(hd->sb_plan[dt == HS_F32 ? 0 : 1]);
+  auto* d = static_cast<sb::DevPlan*>(sb_ten(hd, dt == HS_F32 ? 0 : 1));
   if (!d || !d->ok) return HS_OK;
   const size_t es = dt == HS_F32 ? sizeof(float) : sizeof(double);
   if (((uintptr_t)x % es) != 0 || ((uintptr_t)y % es) != 0) return HS_OK;

@@ -11,6 +11,7 @@
 // a captured CUDA graph, and the host reads the state once per replay to see
 // whether the solve has finished. Same vectors and arithmetic as minres.cu.
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 
 #include "common.cuh"
@@ -74,27 +75,29 @@ hs_status solve_t(hs_handle* hd, const T* b, const MinresVecs& v, double tol, lo
                   bool* used) {
   *used = false;
   const int ti = sizeof(T) == 8 ? 1 : 0;
-  auto* d = static_cast<sb::DevPlan*>(hd->sb_plan[ti]);
-  if (!d || !d->ok) return HS_OK;
-  const sb::Geo& g = d->geo;
-  auto* d4 = static_cast<sb4::DevPlan4*>(hd->sb4_plan[ti]);
-  auto* d6 = static_cast<sb6::DevPlan6*>(hd->sb6_plan);
+  if (!hd->sb_on) return HS_OK;
   const int want = hs_want_sb(sizeof(T) == 8 ? HS_F64 : HS_F32);
-  const bool use4 = want == 4 && d4 && d4->ok;
-  const bool use6 = sizeof(T) == 8 && want == 6 && d6 && d6->ok;
   const auto kA6 = sb6::kernel6<double, sb::MODE_MINRES>();
   // FP32: the class form where the blocks have ten low bits
   const auto kAc = k_cls<sb::MODE_MINRES>;
   const int gc = grid_of(hd, kAc, CLS_NT, 0, CLS_MB * hd->num_sms);
   const bool blk = sizeof(T) == 4 && want == 0;    // element-wise passes of blk_rows.cuh
   const bool cls = blk && hd->d_order && gc >= CLS_CTAS_MIN;
+  // the class form needs no plan
+  auto* d = static_cast<sb::DevPlan*>(cls ? nullptr : sb_ten(hd, ti));
+  if (!cls && (!d || !d->ok)) return HS_OK;
+  const sb::Geo g = d ? d->geo : sb::Geo{};
+  auto* d4 = static_cast<sb4::DevPlan4*>(want == 4 ? sb_four(hd, ti) : nullptr);
+  auto* d6 = static_cast<sb6::DevPlan6*>(hd->sb6_plan);
+  const bool use4 = d4 && d4->ok;
+  const bool use6 = sizeof(T) == 8 && want == 6 && d6 && d6->ok;
   const size_t smA = cls ? 0 : use6 ? d6->smem : use4 ? d4->smem : d->smem;
   const size_t smR = sb::rows_smem_bytes<T>(1 << g.k);
   const int gA = cls ? gc
                : use6 ? grid_of(hd, kA6, sb6::NT6, smA, d6->geo.npairs)
                : use4 ? grid_of(hd, kern_A4<T>(d4->geo.km), nt_a4<T>(), smA, d4->geo.npairs)
                       : grid_of(hd, kern_A<T>(g.km), NT_A, smA, g.npairs);
-  const int gI = grid_of(hd, kern_R<T, PC, sb::ROWS_INIT>(), NT_R, smR, g.npairs);
+  const int gI = blk ? 1 : grid_of(hd, kern_R<T, PC, sb::ROWS_INIT>(), NT_R, smR, g.npairs);
   // FP64: M_ii and its reciprocal kept in memory (without room for them, or for
   // the identity, which needs none, pass B as below)
   constexpr bool flat = sizeof(T) == 8;
@@ -120,7 +123,11 @@ hs_status solve_t(hs_handle* hd, const T* b, const MinresVecs& v, double tol, lo
   ma.m = keeps_m ? hd->sb_m : nullptr;
   ma.mi = ma.m ? hd->sb_m + hd->n : nullptr;
   BlkRows cr{};
-  if (blk) cr = BlkRows{reinterpret_cast<const float*>(b), ma, tol, kmax, hd->d_sigma, g.dscale};
+  if (blk) {
+    double dscale = 0.25 * hd->L;      // as in build_plan (sb.cuh)
+    for (int j = 0; j < hd->L; ++j) dscale += 0.5 * std::fabs(hd->h[j]);
+    cr = BlkRows{reinterpret_cast<const float*>(b), ma, tol, kmax, hd->d_sigma, dscale};
+  }
   // initial pass: q_1 = M^-1 b, beta_1, state
   ma.counter = cr.ma.counter = hd->d_counter + 0;
   if (blk)
