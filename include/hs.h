@@ -71,10 +71,10 @@ typedef struct {
 
 /* Solver forms (all run the recurrence of Algorithm 2): vectors resident on
  * chip (HS_FORM_SMEM: one thread-block cluster for chains of up to 16384 rows,
- * in FP64 up to 4096, else the registers or shared memory of the whole grid,
- * chains up to L = 20 in FP64, 22 in FP32); passes on the blocks and
- * superblocks of long chains (HS_FORM_SUPERBLOCK, from L = 24 on, in FP64 from
- * L = 22 on); one persistent cooperative kernel with vectors in global
+ * in FP64 up to 4096 and with Jacobi up to 16384, else the registers or shared
+ * memory of the whole grid, chains up to L = 20 in FP64, 22 in FP32); passes on
+ * the blocks and superblocks of long chains (HS_FORM_SUPERBLOCK, from L = 24 on;
+ * in FP64 with the identity or the row norm from L = 22 on); one persistent cooperative kernel with vectors in global
  * memory; per-pass kernels replayed from a CUDA graph; and the on-chip form
  * with one global reduction per iteration (the product taken of
  * M^-1 p_k, p carried by the recurrence of q and replaced by a product every
@@ -217,9 +217,10 @@ hs_status hs_eigs_host(int L, const double* h_host, double sigma, int K, int m_m
  * reorthogonalisation; the convergence test on T_k); m (m_max, else
  * max(130, 3K + 30)) is at most 256. Where every chain has at most 4096 rows
  * the groups are thread-block clusters and share one queue, the longest chains
- * first. The group size per (L, pc, SM count) is
+ * first; where the device refuses such clusters, groups of CTAs as for longer
+ * chains. The group size per (L, pc, SM count) is
  * timed on first use and cached in the JSON file HS_SWEEP_TUNE (default
- * $HOME/.cache/hs_sweep_tune.json); HS_SWEEP_S forces it.
+ * $HOME/.cache/hs_sweep_tune.json); HS_SWEEP_S forces groups of that size.
  * Outputs (host, realisation r at offset r K): evals_host (B K, each ordered as
  * by hs_lanczos_eigs and certified the same way), resid_host (B K FP64
  * residuals ||H psi - E psi||, may be NULL), z_host (2 B K: Re, Im of the twist
@@ -336,8 +337,10 @@ hs_status hs_sym_eigvals(int n, double* a_host, double* w_host);
  * may change it while hs_lanczos_eigs runs on this handle: the new share takes
  * effect from the next Lanczos step (for example, to hand the SMs of finished
  * realisations to the ones still running). Keep the shares of concurrent
- * handles summing to at most the SM count. The paper runs one realisation per
- * GPU; this is a throughput setting only. */
+ * handles summing to at most the SM count. The fastest on-chip form needs 39 SMs
+ * at L = 18 and 149 at L = 20 (two-reduction solves); with fewer, a slower one
+ * runs. The paper runs one realisation per GPU; this is a throughput setting
+ * only. */
 hs_status hs_set_sm_budget(hs_handle* hd, int nsm);
 
 /* Number of CUDA kernels this library has launched in the process so far

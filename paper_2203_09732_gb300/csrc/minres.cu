@@ -677,7 +677,8 @@ static int sb_choice(const hs_handle* hd, bool f64, int pc) {
 
 // The one-reduction recurrence is the first choice for FP64 solves with the
 // identity or row-norm preconditioner while a CTA holds at most 1024 rows, in
-// the row layout (minres_row1.cu) where that fits, else minres_pipe.cu: there the
+// the row layout (minres_row1.cu takes up to 1056 rows per CTA); minres_pipe.cu only
+// where that launch is refused, or under HS_MINRES_PIPE=1 with more rows. There the
 // second grid reduction is a third of the iteration (one against two reductions
 // in the row layout, us per iteration on 152 SMs: L = 14 6.0 against 9.6, L = 16
 // 6.3 against 9.6, L = 18 8.9 against 12.4; the same iteration counts, true
@@ -697,11 +698,14 @@ static bool pipe_choice(const hs_handle* hd, bool f64, int pc) {
   return hd->n <= 1024LL * G;
 }
 
-// The cluster form (minres_clu.cu) takes the small solves. Not where another
-// form is asked for (HS_MINRES_PIPE). HS_MINRES_CLUSTER=0 turns it off.
+// The cluster form (minres_clu.cu) takes the small solves: n <= 16384, in FP64 what
+// the one-reduction recurrence does not take above 4096 rows (Jacobi at L = 16: 12.5
+// us per iteration, 18.4 in k_minres_smem, which took it before, 23.1 there on 16
+// SMs; the row form, which is not tried first, 9.6 on the whole GPU). Not where
+// another form is asked for (HS_MINRES_PIPE). HS_MINRES_CLUSTER=0 turns it off.
 static int cluster_choice(const hs_handle* hd, bool f64, int pc) {
   if (getenv("HS_MINRES_PIPE")) return 0;
-  // FP64 above 4096 rows: 16 SMs' FP64 pipes would bound it
+  // FP64 above 4096 rows: 16 SMs' FP64 pipes bound it, the whole grid's do not
   if (f64 && hd->n > CLU_F64_ROWS && pipe_choice(hd, f64, pc)) return 0;
   const int bud = hd->sm_budget.load(std::memory_order_relaxed);
   return clu_choice(hd->n, std::max(1, std::min(hd->num_sms, bud > 0 ? bud : hd->num_sms)));

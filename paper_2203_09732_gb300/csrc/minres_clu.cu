@@ -72,7 +72,8 @@ hs_status launch_rpt(hs_handle* hd, const SmemJob& job, int pc, int cs) {
 //   n = 924    4 CTAs 3.13 / 1.60, 8 CTAs 2.38 / 1.59, 16 CTAs 2.34 / 1.65 (11.7 / 15.6)
 //   n = 3432   8 CTAs 5.4 / 2.4, 16 CTAs 4.12 / 2.16                       (12.2 / 17.1)
 //   n = 12870  16 CTAs FP32 4.98                                            (17.8)
-// FP64 at n = 12870 stays with the grid forms (pipe_choice). HS_MINRES_CLUSTER
+// FP64 at n = 12870 stays with the grid forms where the one-reduction recurrence
+// serves (cluster_choice: Jacobi, 16 CTAs, 12.5 us). HS_MINRES_CLUSTER
 // sets the number of CTAs (a power of two, at most 16; 0: off).
 int clu_choice(long long n, int sms) {
   if (n > CLU_ROWS) return 0;

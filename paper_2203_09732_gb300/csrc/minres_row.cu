@@ -1,7 +1,7 @@
 // Preconditioned MINRES of Algorithm 2 (Appendix A) on the whole GPU with one
-// thread per row (up to four), for chains that a cluster cannot hold and whose
-// neighbour lists fit in shared memory (n up to about 1500 rows per SM: L = 18
-// and 20). One cooperative launch, two reductions per iteration, the arithmetic
+// thread per row (up to three), for chains that a cluster cannot hold and that give
+// a CTA at most 1248 rows (three for each of its 416 compute threads): L = 18 on 39
+// SMs and more, L = 20 on 149 and more; a smaller share takes k_minres_smem. One cooperative launch, two reductions per iteration, the arithmetic
 // of k_minres_smem.
 //
 // What bounded k_minres_smem (38 us per FP64 iteration at n = 184756, 19 of them
@@ -19,7 +19,7 @@
 //     16 to 18 for the longest of 32 rows in rank order);
 //   * in a reduction only CTA 0 reads every CTA's partial sum (grid_total).
 // Per iteration (us, row norm, 152 SMs, before -> here): L = 18 FP64 19.7 (one
-// reduction) -> 11.2, FP32 17.9 -> 8.3; L = 20 FP64 37.7 -> 18.6, FP32 20.1 -> 9.3.
+// reduction) -> 11.4, FP32 17.9 -> 8.3; L = 20 FP64 37.7 -> 18.6, FP32 20.1 -> 10.0.
 // At L = 20 the FP64 pipe takes about 10 us of it (26 instructions a row, 19
 // cycles per warp and SM), the two exchanges about 3 us each.
 #include <algorithm>

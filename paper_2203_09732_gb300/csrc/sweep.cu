@@ -758,8 +758,9 @@ __global__ void __launch_bounds__(CLU_NT, 1) k_sweep_clu(const SweepReal* reals,
 }
 
 // Microseconds per FP64 iteration of n rows on a cluster of cs CTAs: the
-// exchanges and reductions, the rows of a thread, the traffic of q (fitted to
-// the measurements at clu_choice, within 15 %).
+// exchanges and reductions, the rows of a thread, the traffic of q. Against the
+// measurements at clu_choice: within 8 % at n = 924 and 3432, 12 to 17 % too long at
+// n = 252 and 27 % at n = 70; it only ranks cluster sizes.
 double clu_iter_us(long long n, int cs) { return 1.5 + 0.8 * clu_rpt((int)n, cs) + 2.5e-4 * n; }
 
 // The cluster size for a sweep, at least smin: the one whose clusters finish a
