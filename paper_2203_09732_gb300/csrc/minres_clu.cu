@@ -67,11 +67,11 @@ hs_status launch_rpt(hs_handle* hd, const SmemJob& job, int pc, int cs) {
 // CTAs per cluster. More CTAs share the FP64 work but make every exchange
 // longer. Measured per iteration (us, row norm, FP64 / FP32; the grid forms
 // that took these solves before in brackets):
-//   n = 70     1 CTA 1.83 / 1.05, 8 CTAs 1.82 / 1.4                     (12.2 / 15.2)
-//   n = 252    1 CTA 2.73 / 1.38, 2 CTAs 2.10 / 1.35, 8 CTAs 2.02 / 1.48  (11.4 / 15.6)
-//   n = 924    4 CTAs 3.13 / 1.60, 8 CTAs 2.38 / 1.59, 16 CTAs 2.34 / 1.65 (11.7 / 15.6)
-//   n = 3432   8 CTAs 5.4 / 2.4, 16 CTAs 4.12 / 2.16                       (12.2 / 17.1)
-//   n = 12870  16 CTAs FP32 4.98                                            (17.8)
+//   n = 70     1 CTA 1.92 / 1.25, 8 CTAs 1.99 / 1.48                    (12.2 / 15.2)
+//   n = 252    1 CTA 2.74 / 1.35, 2 CTAs 2.16 / 1.35, 8 CTAs 2.09 / 1.48  (11.4 / 15.6)
+//   n = 924    4 CTAs 3.09 / 1.60, 8 CTAs 2.43 / 1.60, 16 CTAs 2.45 / 1.69 (11.7 / 15.6)
+//   n = 3432   8 CTAs 5.46 / 2.29, 16 CTAs 4.04 / 2.19                     (12.2 / 17.1)
+//   n = 12870  16 CTAs FP32 4.78                                            (17.8)
 // FP64 at n = 12870 stays with the grid forms where the one-reduction recurrence
 // serves (cluster_choice: Jacobi, 16 CTAs, 12.5 us). HS_MINRES_CLUSTER
 // sets the number of CTAs (a power of two, at most 16; 0: off).

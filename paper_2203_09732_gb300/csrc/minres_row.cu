@@ -19,7 +19,7 @@
 //     16 to 18 for the longest of 32 rows in rank order);
 //   * in a reduction only CTA 0 reads every CTA's partial sum (grid_total).
 // Per iteration (us, row norm, 152 SMs, before -> here): L = 18 FP64 19.7 (one
-// reduction) -> 11.4, FP32 17.9 -> 8.3; L = 20 FP64 37.7 -> 18.6, FP32 20.1 -> 10.0.
+// reduction) -> 11.4, FP32 17.9 -> 9.0; L = 20 FP64 37.7 -> 18.6, FP32 20.1 -> 10.0.
 // At L = 20 the FP64 pipe takes about 10 us of it (26 instructions a row, 19
 // cycles per warp and SM), the two exchanges about 3 us each.
 #include <algorithm>

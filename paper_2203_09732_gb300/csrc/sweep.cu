@@ -579,9 +579,9 @@ __global__ void __launch_bounds__(NT, 1) k_sweep(SweepArgs a0, SmemQueue q0, Swe
 // Cluster form, for chains of up to CLU_F64_ROWS rows: a thread-block cluster
 // takes a realisation (longest chains first) and runs all of Algorithm 1 on it,
 // the inner solves by clu_solve. 24 chains of L = 10 and 8 of L = 12, 4 pairs
-// each, all calls included: 1063 -> 139 ms (the launch 1009 -> 131 ms: groups of
+// each, all calls included: 1140 -> 154 ms (the launch 1000 -> 132 ms: groups of
 // one CTA were bound by one SM's FP64 pipe, larger ones by the exchange through
-// L2; the setup 126 -> 7 ms: sigma of all chains of a length in one launch).
+// L2; the setup 122 -> 7 ms: sigma of all chains of a length in one launch).
 constexpr int CSW_NW = CLU_NT / 32;
 
 struct CluSweepShared {
@@ -759,8 +759,8 @@ __global__ void __launch_bounds__(CLU_NT, 1) k_sweep_clu(const SweepReal* reals,
 
 // Microseconds per FP64 iteration of n rows on a cluster of cs CTAs: the
 // exchanges and reductions, the rows of a thread, the traffic of q. Against the
-// measurements at clu_choice: within 8 % at n = 924 and 3432, 12 to 17 % too long at
-// n = 252 and 27 % at n = 70; it only ranks cluster sizes.
+// measurements at clu_choice: within 8 % at n = 924 and 3432, 9 to 15 % too long at
+// n = 252 and 21 % at n = 70; it only ranks cluster sizes.
 double clu_iter_us(long long n, int cs) { return 1.5 + 0.8 * clu_rpt((int)n, cs) + 2.5e-4 * n; }
 
 // The cluster size for a sweep, at least smin: the one whose clusters finish a
